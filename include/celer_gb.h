@@ -578,6 +578,13 @@ celer_status celer_debug_curand_philox(uint64_t seed, uint64_t subsequence, uint
  * 1 ulp). fn outside 0-11 or null pointers give CELER_ERR_INVALID. */
 celer_status celer_debug_math(int fn, const double* host_x, uint64_t n, double* host_out);
 
+/* Device arithmetic of the step kernels on n operand pairs: fn 0 the quotient
+ * a / b, 1 the reciprocal 1 / b, 2 the square root of a, 3 the reciprocal
+ * square root of a (Newton-Raphson from the hardware's approximations). No
+ * counterpart in the paper: it checks them against correctly rounded results.
+ * fn outside 0-3 or null pointers give CELER_ERR_INVALID. */
+celer_status celer_debug_arith(int fn, const double* host_a, const double* host_b, uint64_t n, double* host_out);
+
 /* Measure the device's FP64 throughput, the ceiling of the step kernels'
  * arithmetic: blocks_per_sm x (SM count) blocks of 256 threads each run 8
  * independent FP64 fused multiply-add chains for iters iterations, timed

@@ -117,6 +117,7 @@ EXPORTS = [
     "celer_debug_sample", "celer_debug_slots", "celer_set_hit_readout", "celer_set_grid_blocks",
     "celer_set_parent_reuse", "celer_set_async_warps", "celer_debug_barrier_timeout", "celer_debug_queue_wait",
     "celer_debug_tracks", "celer_debug_fp64_rate", "celer_debug_lane_counts",
+    "celer_debug_arith",
 ]
 
 _lib = None
@@ -156,6 +157,7 @@ def load(path: Optional[str] = None):
         "celer_debug_table": ([vp, i32, i32, dp], i32),
         "celer_debug_philox": ([vp, vp, u64], i32),
         "celer_debug_math": ([i32, vp, u64, vp], i32),
+        "celer_debug_arith": ([i32, vp, vp, u64, vp], i32),
         "celer_debug_curand_philox": ([u64, u64, u64, vp, u64], i32),
         "celer_debug_sample": ([i32, u32, u32, vp, C.c_double, vp, vp, u64, vp, vp, vp, vp], i32),
         "celer_debug_slots": ([vp, vp, vp, C.POINTER(i32)], i32),
@@ -559,6 +561,17 @@ def debug_math(fn: int, x: np.ndarray) -> np.ndarray:
     a = np.ascontiguousarray(x, dtype=np.float64)
     out = np.zeros_like(a)
     _check(load().celer_debug_math(int(fn), a.ctypes.data, len(a), out.ctypes.data))
+    return out
+
+
+def debug_arith(fn: int, a: np.ndarray, b: Optional[np.ndarray] = None) -> np.ndarray:
+    """Device arithmetic of the step kernels: 0 a / b, 1 1 / b, 2 sqrt(a),
+    3 1 / sqrt(a)."""
+    a = np.ascontiguousarray(a, dtype=np.float64)
+    b = a if b is None else np.ascontiguousarray(b, dtype=np.float64)
+    assert a.shape == b.shape
+    out = np.zeros_like(a)
+    _check(load().celer_debug_arith(int(fn), a.ctypes.data, b.ctypes.data, len(a), out.ctypes.data))
     return out
 
 

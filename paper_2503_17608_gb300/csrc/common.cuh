@@ -11,6 +11,7 @@ namespace celer {
 constexpr int kGrid = 200;          // log-spaced energy grid points
 constexpr double kGridEmin = 1e-3;  // MeV
 constexpr double kGridEmax = 1e4;   // MeV
+constexpr double kFieldK = 2.99792458;  // curvature [1/cm] = kFieldK * B[T] / p[MeV/c]
 constexpr int kCols = 6;            // device table columns per material
 constexpr int kMaxMaterials = 8;
 constexpr int kMaxLayers = 1024;
@@ -85,8 +86,8 @@ enum ErrorBits : uint32_t { ERR_RING_OVERFLOW = 1u, ERR_NO_PROGRESS = 2u, ERR_IT
 
 struct Tracks {
   double *x, *y, *z, *ux, *uy, *uz, *E, *nmfp, *step, *rpost;
-  double* gfrac;   // a photon's grid position in ln E (bin, fraction), kept
-  int32_t* gbin;   // from the step that sampled its n_mfp (same energy since)
+  double* gfrac;   // the grid position in ln E (bin, fraction) of the track's
+  int32_t* gbin;   // energy, valid while its n_mfp is set
   unsigned long long* tid;
   uint32_t *ctr, *event, *primary;
   int32_t* layer;
@@ -190,6 +191,7 @@ struct Params {
   const double* zb;        // n_layers + 1
   const int32_t* layer_mat;
   double hx, hy, Bz;
+  double field_bk, field_inv_bk;  // Bz times the curvature constant, and its inverse (0 without field)
   // physics
   double cut_track, cut_moller, cut_brems;
   int processes;

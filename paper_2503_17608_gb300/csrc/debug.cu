@@ -59,6 +59,19 @@ __global__ void k_math(int fn, const double* mt, const double* x, double* out, u
 }
 
 
+__global__ void k_arith(int fn, const double* a, const double* b, double* out, uint64_t n) {
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+    double r;
+    switch (fn) {
+      case 0: r = celer::quot(a[i], b[i]); break;
+      case 1: r = celer::recip(b[i]); break;
+      case 2: r = celer::fast_sqrt(a[i]); break;
+      default: r = celer::fast_rsqrt(a[i]); break;
+    }
+    out[i] = r;
+  }
+}
+
 // One rejection sample per record: which 0 the FP32-filtered Compton sampler
 // of the step kernels, 1 its plain FP64 form, 2 the filtered Moller sampler,
 // 3 its plain FP64 form.
@@ -128,6 +141,27 @@ celer_status celer_debug_math(int fn, const double* host_x, uint64_t n, double* 
   cudaFree(d_mt);
   cudaFree(d_x);
   cudaFree(d_out);
+  return st;
+}
+
+celer_status celer_debug_arith(int fn, const double* host_a, const double* host_b, uint64_t n, double* host_out) {
+  if (!host_a || !host_b || !host_out || fn < 0 || fn > 3) return CELER_ERR_INVALID;
+  if (n == 0) return CELER_OK;
+  const size_t bytes = sizeof(double) * n;
+  double* d = nullptr;
+  if (cudaMalloc(&d, 3 * bytes) != cudaSuccess) return CELER_ERR_CUDA;
+  celer_status st = CELER_OK;
+  if (cudaMemcpy(d, host_a, bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(d + n, host_b, bytes, cudaMemcpyHostToDevice) != cudaSuccess)
+    st = CELER_ERR_CUDA;
+  if (st == CELER_OK) {
+    const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
+    k_arith<<<grid, 256>>>(fn, d, d + n, d + 2 * n, n);
+    if (cudaGetLastError() != cudaSuccess ||
+        cudaMemcpy(host_out, d + 2 * n, bytes, cudaMemcpyDeviceToHost) != cudaSuccess)
+      st = CELER_ERR_CUDA;
+  }
+  cudaFree(d);
   return st;
 }
 

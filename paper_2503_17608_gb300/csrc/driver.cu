@@ -447,6 +447,8 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
   p.hx = pb->half_x;
   p.hy = pb->half_y;
   p.Bz = pb->Bz;
+  p.field_bk = pb->Bz * kFieldK;
+  p.field_inv_bk = pb->Bz != 0.0 ? 1.0 / p.field_bk : 0.0;
   p.field_cap = pb->field_substep_cap;
   p.async_warps = 1;  // the asynchronous loop schedules per warp for the block-local policy
   p.cut_track = pb->cut_track;

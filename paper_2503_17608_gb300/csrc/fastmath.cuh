@@ -103,6 +103,86 @@ inline void build_math_table(double* out) {
 }
 
 #ifdef __CUDACC__
+// ---- quotient, square root and reciprocal square root
+//
+// From the hardware's approximation (rcp.approx.ftz.f64, rsqrt.approx.ftz.f64:
+// documented relative error about 2^-23) by Newton-Raphson steps that end in
+// a correction by the exact residual (P. W. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
+// Dev. 34, 1990): the error before the last rounding is below 2^-64, so the
+// quotient and the square root are the correctly rounded ones but for rare
+// near-ties, and the reciprocal square root is within 1 ulp.
+//
+// Why not the operators: they cost 8 to 11 FP64 instructions; these cost 5.
+// On sm_103a an FP64 instruction holds the sub-partition's FP64 pipe for 64
+// cycles and takes five instruction slots of code (80 bytes, measured on the
+// size of compiled loops), and the step loops stall on instruction fetch and
+// on that pipe. Operands outside the middle of the exponent range (zeros,
+// subnormals, infinities and NaN among them) take the operators, one shared
+// copy of each.
+__device__ __forceinline__ double approx_rcp(double b) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+  return r;
+}
+__device__ __forceinline__ double approx_rsqrt(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+// |v| in [2^-510, 2^511), any sign (mid_range) or positive (mid_positive)
+__device__ __forceinline__ bool mid_range(double v) {
+  return (((unsigned)__double2hiint(v) & 0x7FFFFFFFu) - 0x20100000u) < 0x3FC00000u;
+}
+__device__ __forceinline__ bool mid_positive(double v) {
+  return ((unsigned)__double2hiint(v) - 0x20100000u) < 0x3FC00000u;
+}
+static __device__ __noinline__ double quot_any(double n, double b) { return n / b; }
+static __device__ __noinline__ double sqrt_any(double x) { return sqrt(x); }
+static __device__ __noinline__ double rsqrt_any(double x) { return rsqrt(x); }
+
+// 1 / b to about 2^-46 relative: one Newton step.
+__device__ __forceinline__ double rough_rcp(double b) {
+  const double r = approx_rcp(b);
+  return fma(r, fma(-b, r, 1.0), r);
+}
+// n / b given r = 1 / b to a few ulp or better: the rounded quotient.
+__device__ __forceinline__ double quot_by(double n, double b, double r) {
+  const double q = n * r;
+  return fma(fma(-q, b, n), r, q);
+}
+// n / b; |n| at most 2^500 (every dividend of the step kernels is far below).
+__device__ __forceinline__ double quot(double n, double b) {
+  if (!mid_range(b)) return quot_any(n, b);
+  return quot_by(n, b, rough_rcp(b));
+}
+__device__ __forceinline__ double recip(double b) {
+  if (!mid_range(b)) return quot_any(1.0, b);
+  const double r = rough_rcp(b);
+  return fma(r, fma(-b, r, 1.0), r);
+}
+// sqrt x: g -> sqrt x, h -> 1 / (2 sqrt x); the residual x - g^2 is exact
+// enough for the last correction to leave only its rounding.
+__device__ __forceinline__ double fast_sqrt(double x) {
+  if (!mid_positive(x)) return sqrt_any(x);
+  const double y = approx_rsqrt(x);
+  const double g0 = x * y, h = 0.5 * y;
+  const double g = fma(g0, fma(-g0, h, 0.5), g0);
+  return fma(fma(-g, g, x), h, g);
+}
+// 1 / sqrt x: with e = 1 - x y^2, y (1 + e/2 + 3 e^2/8) to O(e^3).
+__device__ __forceinline__ double fast_rsqrt(double x) {
+  if (!mid_positive(x)) return rsqrt_any(x);
+  const double y = approx_rsqrt(x);
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(fma(e, 0.375, 0.5), y * e, y);
+}
+
+// the library's routines for the arguments outside the reduced ranges below,
+// one copy each
+static __device__ __noinline__ double log_any(double x) { return log(x); }
+static __device__ __noinline__ double exp_any(double x) { return exp(x); }
+
 // log x = k ln 2 + L_j + log1p(r), x = 2^k m with m in [0.75, 1.5) taken from
 // the bits (x - bits(0.75) gives k in the exponent field and the interval j
 // in the next 8 bits), r = m / c_j - 1 = fma(m, 1/c_j, -1), |r| < 2^-8.
@@ -112,7 +192,7 @@ inline void build_math_table(double* out) {
 // free for the step code (inlined copies measured 6-9 % slower).
 static __device__ __noinline__ double fast_log(double x, const double* __restrict__ mt) {
   const long long ix = __double_as_longlong(x);
-  if ((unsigned long long)(ix - 0x0010000000000000ll) >= 0x7FE0000000000000ull) return log(x);
+  if ((unsigned long long)(ix - 0x0010000000000000ll) >= 0x7FE0000000000000ull) return log_any(x);
   const long long tmp = ix - 0x3FE8000000000000ll;
   const int k = (int)(tmp >> 52);
   const int j = (int)((tmp >> 44) & (kLogTable - 1));
@@ -139,7 +219,7 @@ static __device__ __noinline__ double fast_log(double x, const double* __restric
 // to the exponent field (|x| < 708 keeps the result normal).
 static __device__ __noinline__ double fast_exp(double x, const double* __restrict__ mt) {
   // |x| < 708 on the bit pattern (NaN and inf fail it, as in FP64)
-  if ((unsigned long long)(__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) >= 0x4086200000000000ull) return exp(x);
+  if ((unsigned long long)(__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) >= 0x4086200000000000ull) return exp_any(x);
   constexpr double kShift = 0x1.8p52;
   const double t = fma(x, __ldg(mt + kMtInvC), kShift);
   const int n = (int)(uint32_t)__double_as_longlong(t);
@@ -162,12 +242,15 @@ static __device__ __noinline__ double fast_exp(double x, const double* __restric
 // tabulated sin, cos of 2 pi j/256 and short Taylor series for theta
 // (truncation below 2^-70). Arguments outside [0, 1] go to sincospi.
 static __device__ __noinline__ void fast_sincos_2pi(double u, const double* __restrict__ mt, double* s, double* c) {
-  if (!(u >= 0.0 && u <= 1.0)) {
+  // 0 <= u <= 1 on the bits (negative, -0 and NaN fall outside)
+  if ((unsigned long long)__double_as_longlong(u) > 0x3FF0000000000000ull) {
     sincospi(2.0 * u, s, c);
     return;
   }
-  const int j = __double2int_rn(u * (double)kSinTable);
-  const double r = u - (double)j * (1.0 / kSinTable);
+  // the nearest integer to 256 u, read from the low bits of 256 u + 1.5 2^52
+  const double t = fma(u, (double)kSinTable, 0x1.8p52);
+  const int j = (int)(uint32_t)__double_as_longlong(t);
+  const double r = fma(t - 0x1.8p52, -1.0 / kSinTable, u);
   const double th = fma(r, __ldg(mt + kMt2PiHi), r * __ldg(mt + kMt2PiLo));
   const double t2 = th * th;
   // sin th = th + th^3 (-1/6 + t2 (1/120 - t2/5040)); cos th - 1 = t2 (-1/2 + t2 (1/24 - t2/720))
@@ -185,12 +268,15 @@ static __device__ __noinline__ void fast_sincos_2pi(double u, const double* __re
 // exact), |r| <= pi/256, then the table and the series of fast_sincos_2pi
 // with theta = r.
 static __device__ __noinline__ void fast_sincos(double x, const double* __restrict__ mt, double* s, double* c) {
-  if (!(fabs(x) < 1e5)) {
+  // |x| < 1e5 on the bits (infinities and NaN fall outside)
+  if ((unsigned long long)(__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) >= 0x40F86A0000000000ull) {
     sincos(x, s, c);
     return;
   }
-  const double jd = rint(x * __ldg(mt + kMtStepInv));
-  const int j = (int)jd;
+  // the nearest integer to x 256 / 2 pi, read from the low bits
+  const double t = fma(x, __ldg(mt + kMtStepInv), 0x1.8p52);
+  const double jd = t - 0x1.8p52;
+  const int j = (int)(uint32_t)__double_as_longlong(t);
   const double th = fma(-jd, __ldg(mt + kMtStepLo), fma(-jd, __ldg(mt + kMtStepHi), x));
   const double t2 = th * th;
   const double sp = fma(t2, fma(t2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0);

@@ -18,7 +18,6 @@ namespace celer {
 constexpr double kMe = 0.51099895;        // electron mass, MeV
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kTwoPi = 2.0 * kPi;
-constexpr double kFieldK = 2.99792458;    // curvature [1/cm] = kFieldK * B[T] / p[MeV/c]
 constexpr double kPairThreshold = 1.022;  // MeV, as in the photon model definition
 constexpr double kAlphaR = 0.2;           // range step function: fraction of range
 constexpr double kFinalR = 0.1;           // range step function: final range, cm
@@ -35,6 +34,7 @@ constexpr int kMaxCasAttempts = 1 << 16;
 // more roundings).
 constexpr double kLimitMargin = 1.0 + 0x1p-50;
 constexpr double kRangeMargin = 1.0 + 0x1p-48;
+constexpr long long kLimitUlps = 8;  // the same for nmfp / mu tested as nmfp <= s mu, on the bits
 // Longest wait at a grid barrier of the persistent loop (~1 s at 2 GHz).
 constexpr long long kBarrierTimeoutCycles = 2000000000ll;
 
@@ -101,6 +101,8 @@ struct TrackRng {
 // states why its operands qualify and why a NaN gives the outcome of the
 // FP64 comparison.
 __device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+// a > b for b >= +0 (a of any sign; a positive NaN counts as greater).
+__device__ __forceinline__ bool farther(double a, double b) { return dbits(a) > dbits(b); }
 
 // ------------------------------------------------------------------ tables
 struct GridPos {
@@ -126,8 +128,9 @@ __device__ __forceinline__ double interp(const double2* col, GridPos g) {
 // R_i <= r, then ln E linear in R inside it. r <= R_0: the track stopped.
 // Ranges are non-negative, so the search compares their bit patterns as
 // integers (same order as the values) and keeps the FP64 pipe free.
+// g receives the grid position of the result: ln E is formed from it.
 __device__ __forceinline__ double inverse_range(const double2* R, double r, double lnEmin, double dl,
-                                                const double* mt) {
+                                                const double* mt, GridPos& g) {
   const long long rb = __double_as_longlong(r);
   if (rb <= __double_as_longlong(R[0].x)) return 0.0;  // r <= R_0 > 0 on the bits (r may be negative)
   int lo = 0;
@@ -137,8 +140,8 @@ __device__ __forceinline__ double inverse_range(const double2* R, double r, doub
     if (probe <= kGrid - 2 && __double_as_longlong(R[probe].x) <= rb) lo = probe;
   }
   const double2 v = R[lo];
-  const double lnE = lnEmin + lo * dl + (r - v.x) / v.y * dl;
-  return fast_exp(lnE, mt);
+  g = GridPos{lo, quot(r - v.x, v.y)};
+  return fast_exp(fma((double)lo, dl, lnEmin) + g.frac * dl, mt);
 }
 
 // ------------------------------------------------------------- kinematics
@@ -148,37 +151,35 @@ __device__ __forceinline__ double inverse_range(const double2* R, double r, doub
 
 // Rotate (ux, uy, uz) by polar cosine cost and azimuth 2 pi u_phi about
 // itself: frame e1 = (u x z)/|u x z|, e2 = u x e1 (e1 = x near the poles),
-// then renormalised. The input is a unit vector to rounding, so the result's
-// squared norm q is 1 + O(1e-16) and one Newton step from 1, 1.5 - q/2, is
-// 1/sqrt(q) to O((q - 1)^2).
+// then renormalised. With n = |u x z|, q = n^2 and w = sin(theta)/n =
+// t rsqrt(t q), t = 1 - cost^2 (one reciprocal square root for the sine and
+// the frame), A = w cos(phi), B = w sin(phi):
+//   v = (C ux + A uy, C uy - A ux, cost uz - B q), C = cost + B uz.
+// The input is a unit vector to rounding, so the result's squared norm is
+// 1 + O(1e-16) and one Newton step from 1, 1.5 - |v|^2/2, is its reciprocal
+// square root to O((|v|^2 - 1)^2).
 __device__ __forceinline__ void rotate_dir(double& ux, double& uy, double& uz, double cost, double u_phi,
                                            const double* mt) {
-  const double sint = sqrt(fmax(0.0, 1.0 - cost * cost));
+  double t = fma(-cost, cost, 1.0);
+  if (dbits(t) < 0) t = 0.0;
   double sp, cp;
   fast_sincos_2pi(u_phi, mt, &sp, &cp);
-  double e1x, e1y, e1z, e2x, e2y, e2z;
+  double vx, vy, vz;
   if ((dbits(uz) & 0x7FFFFFFFFFFFFFFFll) < dbits(1.0 - 1e-10)) {  // |uz| < 1 - 1e-10 on the bits
-    const double q = ux * ux + uy * uy;
-    const double inv_n = rsqrt(q);
-    e1x = uy * inv_n;
-    e1y = -ux * inv_n;
-    e1z = 0.0;
-    e2x = uz * ux * inv_n;
-    e2y = uz * uy * inv_n;
-    e2z = -q * inv_n;
+    const double q = fma(ux, ux, uy * uy);
+    const double w = dbits(t) != 0 ? t * fast_rsqrt(t * q) : 0.0;
+    const double A = w * cp, B = w * sp;
+    const double C = fma(B, uz, cost);
+    vx = fma(C, ux, A * uy);
+    vy = fma(C, uy, -A * ux);
+    vz = fma(cost, uz, -B * q);
   } else {
-    const double q = uz * uz + uy * uy;
-    const double inv_n = rsqrt(q);
-    e1x = 1.0;
-    e1y = 0.0;
-    e1z = 0.0;
-    e2x = 0.0;
-    e2y = uz * inv_n;
-    e2z = -uy * inv_n;
+    const double sint = fast_sqrt(t);
+    const double B = sint * sp * fast_rsqrt(fma(uz, uz, uy * uy));
+    vx = fma(cost, ux, sint * cp);
+    vy = fma(cost, uy, B * uz);
+    vz = fma(cost, uz, -B * uy);
   }
-  const double vx = cost * ux + sint * (cp * e1x + sp * e2x);
-  const double vy = cost * uy + sint * (cp * e1y + sp * e2y);
-  const double vz = cost * uz + sint * (cp * e1z + sp * e2z);
   const double inv = fma(-0.5, fma(vx, vx, fma(vy, vy, vz * vz)), 1.5);
   ux = vx * inv;
   uy = vy * inv;
@@ -191,12 +192,12 @@ __device__ __forceinline__ void rotate_dir(double& ux, double& uy, double& uz, d
 struct Curvature {
   double kappa, inv_kappa;
 };
-__device__ __forceinline__ Curvature curvature(uint8_t ptype, double E, double Bz) {
-  const double q = (ptype == ELECTRON) ? -1.0 : 1.0;
+__device__ __forceinline__ Curvature curvature(const Params& p, uint8_t ptype, double E) {
+  const double bk = (ptype == ELECTRON) ? -p.field_bk : p.field_bk;
+  const double inv = (ptype == ELECTRON) ? -p.field_inv_bk : p.field_inv_bk;
   const double p2 = E * (E + 2.0 * kMe);
-  const double r = rsqrt(p2);
-  const double qbk = q * Bz * kFieldK;
-  return Curvature{qbk * r, (p2 * r) / qbk};
+  const double r = fast_rsqrt(p2);
+  return Curvature{bk * r, quot_by(p2 * r, bk, inv)};
 }
 
 // Exact helix for du/ds = kappa (u x z), with 1 - cos(phi) = 2 sin^2(phi/2).
@@ -224,13 +225,14 @@ __device__ __forceinline__ void helix_move(Curvature c, double s, double& x, dou
 // length at the start.
 constexpr double kRkTurn = 0.1;
 __device__ __forceinline__ int rk_substeps(double kappa, double s) {
-  const int n = (int)ceil(s * fabs(kappa) / kRkTurn);
+  const int n = (int)ceil(quot_by(s * fabs(kappa), kRkTurn, 1.0 / kRkTurn));
   return n < 1 ? 1 : n;
 }
 __device__ __forceinline__ void rk_move(double kappa, double s, int n, double& x, double& y, double& z, double& ux,
                                         double& uy, double uz) {
   const double q0 = ux * ux + uy * uy;
-  const double h = s / n;
+  const double h = quot(s, (double)n);
+  const double h6 = quot_by(h, 6.0, 1.0 / 6.0);
   double X = x, Y = y, U = ux, V = uy;
   for (int i = 0; i < n; ++i) {
     const double c1 = kappa * V, d1 = -kappa * U;
@@ -240,14 +242,14 @@ __device__ __forceinline__ void rk_move(double kappa, double s, int n, double& x
     const double c3 = kappa * V3, d3 = -kappa * U3;
     const double U4 = U + h * c3, V4 = V + h * d3;
     const double c4 = kappa * V4, d4 = -kappa * U4;
-    X += h / 6.0 * (U + 2.0 * U2 + 2.0 * U3 + U4);
-    Y += h / 6.0 * (V + 2.0 * V2 + 2.0 * V3 + V4);
-    U += h / 6.0 * (c1 + 2.0 * c2 + 2.0 * c3 + c4);
-    V += h / 6.0 * (d1 + 2.0 * d2 + 2.0 * d3 + d4);
+    X += h6 * (U + 2.0 * U2 + 2.0 * U3 + U4);
+    Y += h6 * (V + 2.0 * V2 + 2.0 * V3 + V4);
+    U += h6 * (c1 + 2.0 * c2 + 2.0 * c3 + c4);
+    V += h6 * (d1 + 2.0 * d2 + 2.0 * d3 + d4);
   }
   const double q = U * U + V * V;
   if (q > 0.0) {
-    const double f = sqrt(q0 / q);
+    const double f = fast_sqrt(quot(q0, q));
     U *= f;
     V *= f;
   }
@@ -277,7 +279,7 @@ static __device__ __noinline__ double helix_side_distance(Curvature c, double x,
   CELER_LANES(LS_HELIX_SIDE);
   const double A2 = ux * ux + uy * uy;
   if (dbits(A2) == 0ll) return kInf;  // A2 >= +0
-  const double inv_A = rsqrt(A2);
+  const double inv_A = fast_rsqrt(A2);
   const double A = A2 * inv_A;
   const double kappa = c.kappa;
   const double inv_K = fabs(c.inv_kappa);
@@ -359,8 +361,8 @@ __device__ __forceinline__ float f32_trunc(double v) {
 // gives the same results with FP32 filtering.
 static __device__ __noinline__ double sample_compton_fp64(double E, TrackRng& rng, double& cost, bool& ok,
                                                           const double* mt) {
-  const double k = E / kMe;
-  const double eps0 = 1.0 / (1.0 + 2.0 * k);
+  const double k = quot_by(E, kMe, 1.0 / kMe);
+  const double eps0 = recip(fma(2.0, k, 1.0));
   const double eps0sq = eps0 * eps0;
   const double a1 = -fast_log(eps0, mt);
   const double w = 1.0 - eps0sq;
@@ -373,13 +375,13 @@ static __device__ __noinline__ double sample_compton_fp64(double E, TrackRng& rn
     if (u1 * (a1 + 0.5 * w) < a1) {
       eps = fast_exp(-a1 * u2, mt);
     } else {
-      eps = sqrt(fma(w, u2, eps0sq));
+      eps = fast_sqrt(fma(w, u2, eps0sq));
     }
     const double a = 1.0 - eps;
     const double b = k * eps;
     const double B = b * b * (1.0 + eps * eps);
     if (eps * a * (2.0 * b - a) <= (1.0 - u3) * B) {
-      t = a / b;
+      t = quot(a, b);
       ok = true;
       break;
     }
@@ -402,11 +404,11 @@ static __device__ __noinline__ double sample_compton_fp64(double E, TrackRng& rn
 // the loop, lanes accepting at different attempts would each run it).
 static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, double& cost, bool& ok,
                                                      const double* mt) {
-  const double k = E / kMe;
+  const double k = quot_by(E, kMe, 1.0 / kMe);
   // 1e-4 <= k <= 1e6 on the bits (negative and NaN k fall outside)
   if ((unsigned long long)(dbits(k) - dbits(1e-4)) > (unsigned long long)(dbits(1e6) - dbits(1e-4)))
     return sample_compton_fp64(E, rng, cost, ok, mt);
-  const double eps0 = 1.0 / (1.0 + 2.0 * k);
+  const double eps0 = recip(fma(2.0, k, 1.0));
   const double eps0sq = eps0 * eps0;
   const double a1 = -fast_log(eps0, mt);
   const double w = 1.0 - eps0sq;
@@ -461,7 +463,7 @@ static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, do
     if (verdict < 0) {  // the plain FP64 attempt
       const double u2 = unit_from_bits(w2);
       if (branch == 0) branch = (unit_from_bits(w1) * (a1 + 0.5 * w) < a1) ? 1 : 2;
-      const double e = branch == 1 ? fast_exp(-a1 * u2, mt) : sqrt(fma(w, u2, eps0sq));
+      const double e = branch == 1 ? fast_exp(-a1 * u2, mt) : fast_sqrt(fma(w, u2, eps0sq));
       const double a = 1.0 - e;
       const double b = k * e;
       const double B = b * b * (1.0 + e * e);
@@ -475,8 +477,8 @@ static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, do
   double eps = 1.0, t = 0.0;
   if (ok) {
     const double u2 = unit_from_bits(w2_acc);
-    eps = branch_acc == 1 ? fast_exp(-a1 * u2, mt) : sqrt(fma(w, u2, eps0sq));
-    t = (1.0 - eps) / (k * eps);
+    eps = branch_acc == 1 ? fast_exp(-a1 * u2, mt) : fast_sqrt(fma(w, u2, eps0sq));
+    t = quot(1.0 - eps, k * eps);
   }
   cost = 1.0 - t;
   return eps;
@@ -487,17 +489,17 @@ static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, do
 // The test u2 <= norm f(eps) is taken multiplied by the positive (1 - eps)^2.
 // Plain FP64 form; sample_moller below gives the same results.
 static __device__ __noinline__ double sample_moller_fp64(double T, double Tcut, TrackRng& rng, bool& ok) {
-  const double x = Tcut / T;
+  const double x = quot(Tcut, T);
   const double y = 1.0 - 2.0 * x;
-  const double g = T / kMe + 1.0;
+  const double g = quot_by(T, kMe, 1.0 / kMe) + 1.0;
   const double g2 = g * g;
-  const double norm = 4.0 / (9.0 * g2 - 10.0 * g + 5.0);
+  const double norm = quot(4.0, 9.0 * g2 - 10.0 * g + 5.0);
   ok = false;
   double eps = 0.5;
   for (int attempt = 0; attempt < kMaxAttempts; ++attempt) {
     const double u1 = rng.uniform();
     const double u2 = rng.uniform();
-    eps = x / fma(-u1, y, 1.0);
+    eps = quot(x, fma(-u1, y, 1.0));
     const double om = 1.0 - eps;
     const double eom = eps * om;
     const double fom2 = (g - 1.0) * (g - 1.0) * eom * eom - (2.0 * g2 + 2.0 * g - 1.0) * eom + g2;
@@ -518,7 +520,7 @@ static __device__ __noinline__ double sample_moller_fp64(double T, double Tcut, 
 // g, g^2 and the normalisation are needed in FP64 only for an undecided
 // attempt; the accepted attempt's eps is computed once, after the loop.
 static __device__ __noinline__ double sample_moller(double T, double Tcut, TrackRng& rng, bool& ok) {
-  const double x = Tcut / T;
+  const double x = quot(Tcut, T);
   // 1e-8 <= x < 1/2 on the bits (negative and NaN x fall outside)
   if ((unsigned long long)(dbits(x) - dbits(1e-8)) >= (unsigned long long)(dbits(0.5) - dbits(1e-8)))
     return sample_moller_fp64(T, Tcut, rng, ok);
@@ -557,12 +559,12 @@ static __device__ __noinline__ double sample_moller(double T, double Tcut, Track
     if (verdict == 0) continue;
     if (verdict < 0) {  // the plain FP64 attempt
       if (!fp64_ready) {
-        g = T / kMe + 1.0;
+        g = quot_by(T, kMe, 1.0 / kMe) + 1.0;
         g2 = g * g;
-        norm = 4.0 / (9.0 * g2 - 10.0 * g + 5.0);
+        norm = quot(4.0, 9.0 * g2 - 10.0 * g + 5.0);
         fp64_ready = true;
       }
-      const double e = x / fma(-unit_from_bits(w1), y, 1.0);
+      const double e = quot(x, fma(-unit_from_bits(w1), y, 1.0));
       const double om = 1.0 - e;
       const double eom = e * om;
       const double fom2 = (g - 1.0) * (g - 1.0) * eom * eom - (2.0 * g2 + 2.0 * g - 1.0) * eom + g2;
@@ -572,7 +574,7 @@ static __device__ __noinline__ double sample_moller(double T, double Tcut, Track
     ok = true;
     break;
   }
-  return ok ? x / fma(-unit_from_bits(w1_acc), y, 1.0) : 0.5;
+  return ok ? quot(x, fma(-unit_from_bits(w1_acc), y, 1.0)) : 0.5;
 }
 
 }  // namespace celer

@@ -198,16 +198,16 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
   const double2* mt = tab + lmat[layer] * (kCols * kGrid);
   const bool charged = pt != GAMMA;
   if (!charged) CELER_LANE_MARK(LS_T_LIMIT, t_mark);
-  // A photon's energy changes only where its n_mfp is reset (creation, an
-  // interaction), so the grid position computed at the step that samples
-  // n_mfp holds until the next such step: later steps reload it.
+  // The grid position of E: computed at the step that samples n_mfp and kept
+  // in the slot. A photon's energy changes only where n_mfp is reset
+  // (creation, an interaction); a charged track's continuous loss forms its
+  // new energy from its new grid position, which the along-step keeps. So
+  // later steps reload it instead of taking the logarithm.
   GridPos g;
-  if (charged || fresh) {
+  if (fresh) {
     g = grid_pos(E, p.lnEmin, p.inv_dl, p.mtab);
-    if (!charged) {
-      t.gbin[slot] = g.bin;
-      t.gfrac[slot] = g.frac;
-    }
+    t.gbin[slot] = g.bin;
+    t.gfrac[slot] = g.frac;
   } else {
     g = GridPos{gbin, gfrac};
   }
@@ -240,7 +240,7 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
   const unsigned long long uza = (unsigned long long)uzb & 0x7FFFFFFFFFFFFFFFull;
   if (uza != 0ull && uza <= 0x7FF0000000000000ull) {  // uz nonzero, not NaN: one division whatever the sign
     const bool up = uzb >= 0;
-    s_geo = (zb[up ? layer + 1 : layer] - z) / uz;
+    s_geo = quot(zb[up ? layer + 1 : layer] - z, uz);
     act = up ? A_ZUP : A_ZDOWN;
   }
   double s_side = kInf;
@@ -252,8 +252,8 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
     // cannot be the shorter one, and is not computed (+4 % on the 4 T
     // calorimeter, whose high-energy circles all cross the side planes).
     const double reach = s_geo + 1e-3;
-    if (!(p.hx - fabs(x) > reach && p.hy - fabs(y) > reach))
-      s_side = helix_side_distance(curvature(pt, E, p.Bz), x, y, ux, uy, p.hx, p.hy);
+    if (!(farther(p.hx - fabs(x), reach) && farther(p.hy - fabs(y), reach)))
+      s_side = helix_side_distance(curvature(p, pt, E), x, y, ux, uy, p.hx, p.hy);
   } else {
     const double reach = s_geo * kLimitMargin;
     // both planes beyond reach along their axis (|u| <= 1 + 2^-52, hence
@@ -266,11 +266,11 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
       const long long bx = dbits(ux), by = dbits(uy);
       if (((unsigned long long)bx << 1) != 0ull) {
         const double d = bx > 0 ? p.hx - x : -p.hx - x;
-        if ((bx > 0 ? d : -d) <= reach * fabs(ux)) s_side = d / ux;
+        if ((bx > 0 ? d : -d) <= reach * fabs(ux)) s_side = quot(d, ux);
       }
       if (((unsigned long long)by << 1) != 0ull) {
         const double d = by > 0 ? p.hy - y : -p.hy - y;
-        if ((by > 0 ? d : -d) <= reach * fabs(uy)) s_side = fmin(s_side, d / uy);
+        if ((by > 0 ? d : -d) <= reach * fabs(uy)) s_side = fmin(s_side, quot(d, uy));
       }
     }
   }
@@ -291,7 +291,7 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
     if (dbits(R) <= dbits(kFinalR)) {
       s_rng = R;
     } else if (dbits(kAlphaR * R + kFinalR * (1.0 - kAlphaR)) <= dbits(s * kRangeMargin)) {
-      s_rng = kAlphaR * R + kFinalR * (1.0 - kAlphaR) * (2.0 - kFinalR / R);
+      s_rng = kAlphaR * R + kFinalR * (1.0 - kAlphaR) * (2.0 - quot(kFinalR, R));
     }
     if (dbits(s_rng) < dbits(s)) {  // s_rng >= +0; s >= +0 or -0 (then false either way)
       s = s_rng;
@@ -300,9 +300,11 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
   }
   bool interact = false;
   // mu > 0 on the bits (mu >= +0: a sum of interpolated non-negative
-  // tables; for a NaN mu the second test fails either way)
-  if (dbits(mu) > 0 && nmfp <= s * mu * kLimitMargin) {
-    const double s_int = nmfp / mu;
+  // tables); the quotient nmfp / mu can be below s only if nmfp is below
+  // s mu (rounded) by the bits or within a few ulp of it (both >= +0; for a
+  // NaN product the quotient is NaN and fails the test after)
+  if (dbits(mu) > 0 && dbits(nmfp) <= dbits(s * mu) + kLimitUlps) {
+    const double s_int = quot(nmfp, mu);
     if (dbits(s_int) < dbits(s)) {  // s_int >= +0; s >= +0 or -0 (then false either way)
       s = s_int;
       interact = true;
@@ -316,9 +318,9 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
     // needing more than `cap` substeps of 0.1 rad of turn is cut there and
     // ends without a crossing or an interaction, to go on next iteration
     if (helix && p.field_cap > 0) {
-      const double kappa = curvature(pt, E, p.Bz).kappa;
+      const double kappa = curvature(p, pt, E).kappa;
       if (s * fabs(kappa) > kRkTurn * p.field_cap) {
-        s = kRkTurn * p.field_cap / fabs(kappa);
+        s = quot(kRkTurn * p.field_cap, fabs(kappa));
         act = A_FIELD;
         interact = false;
       }
@@ -851,7 +853,7 @@ __device__ __forceinline__ bool along_one(const Params& p, uint32_t slot, uint8_
   const bool eloss = charged && (p.processes & PROC_ELOSS);
   const bool helix = charged && ((unsigned long long)dbits(p.Bz) << 1) != 0ull;  // Bz != 0 on the bits
   if (helix) {
-    const Curvature cv = curvature(pt, E, p.Bz);
+    const Curvature cv = curvature(p, pt, E);
     if (p.field_cap > 0)
       rk_move(cv.kappa, s, act == A_FIELD ? p.field_cap : rk_substeps(cv.kappa, s), x, y, z, ux, uy, uz);
     else
@@ -863,7 +865,10 @@ __device__ __forceinline__ bool along_one(const Params& p, uint32_t slot, uint8_
   }
   if (eloss) {
     const double2* R = ss.tab + (ss.lmat[layer] * kCols + COL_RANGE) * kGrid;
-    const double Ep = inverse_range(R, t.rpost[slot], p.lnEmin, p.dl, p.mtab);
+    GridPos g{0, 0.0};
+    const double Ep = inverse_range(R, t.rpost[slot], p.lnEmin, p.dl, p.mtab, g);
+    t.gbin[slot] = g.bin;
+    t.gfrac[slot] = g.frac;
     deposit(p, ev, prim, layer, z, E - Ep);
     E = Ep;
   }
@@ -1051,7 +1056,8 @@ __device__ __forceinline__ bool pair_one(const Params& p, uint32_t slot, uint8_t
   deposit(p, ev, prim, layer, z, E - 2.0 * kMe);
   const double cost = 2.0 * rng.uniform() - 1.0;
   const double u_phi = rng.uniform();
-  const double sint = sqrt(fmax(0.0, 1.0 - cost * cost));
+  const double sint2 = 1.0 - cost * cost;
+  const double sint = dbits(sint2) > 0 ? fast_sqrt(sint2) : 0.0;
   double sp_, cp_;
   fast_sincos_2pi(u_phi, p.mtab, &sp_, &cp_);
   const double dx = sint * cp_, dy = sint * sp_, dz = cost;
@@ -1123,7 +1129,7 @@ __device__ __forceinline__ bool moller_one(const Params& p, uint32_t slot, uint8
   // sqrt(Td (T + 2m) / (T (Td + 2m))) = Td (T + 2m) / (p p_delta), from two
   // reciprocal square roots
   const double pp2 = T * (T + 2.0 * kMe), pd2 = Td * (Td + 2.0 * kMe);
-  const double rpp = rsqrt(pp2), rpd = rsqrt(pd2);
+  const double rpp = fast_rsqrt(pp2), rpd = fast_rsqrt(pd2);
   const double cost = fmin(1.0, Td * (T + 2.0 * kMe) * rpp * rpd);
   const double u_phi = rng.uniform();
   const double ux = t.ux[slot], uy = t.uy[slot], uz = t.uz[slot];
@@ -1132,7 +1138,7 @@ __device__ __forceinline__ bool moller_one(const Params& p, uint32_t slot, uint8
   const double pp = pp2 * rpp;
   const double pd = pd2 * rpd;
   const double vx = pp * ux - pd * dx, vy = pp * uy - pd * dy, vz = pp * uz - pd * dz;
-  const double inv = rsqrt(vx * vx + vy * vy + vz * vz);
+  const double inv = fast_rsqrt(vx * vx + vy * vy + vz * vz);
   const double E1 = T - Td;
   if (keep) {
     const unsigned long long tid = rng.raw();
@@ -1171,7 +1177,7 @@ __device__ __forceinline__ bool brems_one(const Params& p, uint32_t slot, uint8_
   }
   const uint32_t ev = t.event[slot], prim = t.primary[slot];
   TrackRng rng(p.seed, ev, t.tid[slot], t.ctr[slot]);
-  double k = p.cut_brems * fast_exp(rng.uniform() * fast_log(T / p.cut_brems, p.mtab), p.mtab);
+  double k = p.cut_brems * fast_exp(rng.uniform() * fast_log(quot(T, p.cut_brems), p.mtab), p.mtab);
   if (k > T) k = T;
   const bool keep = k >= p.cut_track;
   unsigned long long base;
