@@ -315,29 +315,13 @@ struct PassCounts {
 // the slot vacant; the run then ends with ERR_BARRIER_TIMEOUT.
 template <bool kAsync>
 __device__ __forceinline__ void take_initializer(const Params& p, unsigned long long index, uint32_t slot) {
-  const Tracks& t = p.trk;
   const unsigned long long i = index & p.ring_mask;
   unsigned code = 0;
   if (kAsync) {
     code = ring_lap_code(p, index) + 1u;
     if (!ring_wait(p, index, code)) return;
   }
-  t.x[slot] = __ldcg(&p.ring.x[i]);
-  t.y[slot] = __ldcg(&p.ring.y[i]);
-  t.z[slot] = __ldcg(&p.ring.z[i]);
-  t.ux[slot] = __ldcg(&p.ring.ux[i]);
-  t.uy[slot] = __ldcg(&p.ring.uy[i]);
-  t.uz[slot] = __ldcg(&p.ring.uz[i]);
-  t.E[slot] = __ldcg(&p.ring.E[i]);
-  t.tid[slot] = __ldcg(&p.ring.tid[i]);
-  t.event[slot] = __ldcg(&p.ring.event[i]);
-  t.primary[slot] = __ldcg(&p.ring.primary[i]);
-  t.layer[slot] = __ldcg(&p.ring.layer[i]);
-  t.ptype[slot] = __ldcg(&p.ring.ptype[i]);
-  t.ctr[slot] = 0u;
-  t.nmfp[slot] = -1.0;
-  t.action[slot] = A_NONE;
-  t.status[slot] = ALIVE;
+  fill_slot(p, slot, get_record(p.ring.rec + i));
   if (kAsync) st_release_u32(p.ring_state + i, code + 1u);
 }
 
@@ -376,7 +360,7 @@ __device__ void data_pass(const Params& p, int bid, int nb, const SharedStatic& 
     bool neutral = false;
     if (in) {
       if (!kAsync || ring_wait(p, first + e, ring_lap_code(p, first + e) + 1u))
-        neutral = __ldcg(&p.ring.ptype[(first + e) & p.ring_mask]) == GAMMA;
+        neutral = __ldcg(&p.ring.rec[(first + e) & p.ring_mask].ptype) == GAMMA;
     }
     unsigned round_n = 0;
     const unsigned rn = n_neutral + block_exclusive_scan(neutral ? 1u : 0u, round_n);

@@ -94,12 +94,18 @@ struct Tracks {
   uint8_t *ptype, *status, *action, *key;
 };
 
+// One entry of the initializer buffer: 80 bytes, moved as five 16-byte parts
+// with one address (an array per field took an address and an access each).
+struct __align__(16) InitRecord {
+  double x, y, z, ux, uy, uz, E;
+  unsigned long long tid;
+  uint32_t event, primary;
+  int32_t layer;
+  uint32_t ptype;
+};
+static_assert(sizeof(InitRecord) == 80, "five 16-byte parts");
 struct Ring {
-  double *x, *y, *z, *ux, *uy, *uz, *E;
-  unsigned long long* tid;
-  uint32_t *event, *primary;
-  int32_t* layer;
-  uint8_t* ptype;
+  InitRecord* rec;
 };
 
 // Device-resident loop control. Ring indices are monotonic counters; the

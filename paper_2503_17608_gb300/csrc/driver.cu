@@ -488,19 +488,7 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
   CREATE_CUDA(dalloc(ctx, &t.status, N));
   CREATE_CUDA(dalloc(ctx, &t.action, N));
   CREATE_CUDA(dalloc(ctx, &t.key, N));
-  Ring& r = p.ring;
-  CREATE_CUDA(dalloc(ctx, &r.x, C));
-  CREATE_CUDA(dalloc(ctx, &r.y, C));
-  CREATE_CUDA(dalloc(ctx, &r.z, C));
-  CREATE_CUDA(dalloc(ctx, &r.ux, C));
-  CREATE_CUDA(dalloc(ctx, &r.uy, C));
-  CREATE_CUDA(dalloc(ctx, &r.uz, C));
-  CREATE_CUDA(dalloc(ctx, &r.E, C));
-  CREATE_CUDA(dalloc(ctx, &r.tid, C));
-  CREATE_CUDA(dalloc(ctx, &r.event, C));
-  CREATE_CUDA(dalloc(ctx, &r.primary, C));
-  CREATE_CUDA(dalloc(ctx, &r.layer, C));
-  CREATE_CUDA(dalloc(ctx, &r.ptype, C));
+  CREATE_CUDA(dalloc(ctx, &p.ring.rec, C));
   CREATE_CUDA(dalloc(ctx, &p.ctl, 1));
   p.n_chunks = (N + 31) / 32;
   CREATE_CUDA(dalloc(ctx, &p.vacant, p.n_chunks));

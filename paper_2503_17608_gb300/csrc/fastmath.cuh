@@ -182,6 +182,8 @@ __device__ __forceinline__ double fast_rsqrt(double x) {
 // one copy each
 static __device__ __noinline__ double log_any(double x) { return log(x); }
 static __device__ __noinline__ double exp_any(double x) { return exp(x); }
+static __device__ __noinline__ void sincos_any(double x, double* s, double* c) { sincos(x, s, c); }
+static __device__ __noinline__ void sincospi_any(double x, double* s, double* c) { sincospi(x, s, c); }
 
 // log x = k ln 2 + L_j + log1p(r), x = 2^k m with m in [0.75, 1.5) taken from
 // the bits (x - bits(0.75) gives k in the exponent field and the interval j
@@ -244,7 +246,7 @@ static __device__ __noinline__ double fast_exp(double x, const double* __restric
 static __device__ __noinline__ void fast_sincos_2pi(double u, const double* __restrict__ mt, double* s, double* c) {
   // 0 <= u <= 1 on the bits (negative, -0 and NaN fall outside)
   if ((unsigned long long)__double_as_longlong(u) > 0x3FF0000000000000ull) {
-    sincospi(2.0 * u, s, c);
+    sincospi_any(2.0 * u, s, c);
     return;
   }
   // the nearest integer to 256 u, read from the low bits of 256 u + 1.5 2^52
@@ -270,7 +272,7 @@ static __device__ __noinline__ void fast_sincos_2pi(double u, const double* __re
 static __device__ __noinline__ void fast_sincos(double x, const double* __restrict__ mt, double* s, double* c) {
   // |x| < 1e5 on the bits (infinities and NaN fall outside)
   if ((unsigned long long)(__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) >= 0x40F86A0000000000ull) {
-    sincos(x, s, c);
+    sincos_any(x, s, c);
     return;
   }
   // the nearest integer to x 256 / 2 pi, read from the low bits

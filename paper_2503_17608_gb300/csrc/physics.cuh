@@ -228,8 +228,11 @@ __device__ __forceinline__ int rk_substeps(double kappa, double s) {
   const int n = (int)ceil(quot_by(s * fabs(kappa), kRkTurn, 1.0 / kRkTurn));
   return n < 1 ? 1 : n;
 }
-__device__ __forceinline__ void rk_move(double kappa, double s, int n, double& x, double& y, double& z, double& ux,
-                                        double& uy, double uz) {
+struct RkState {
+  double x, y, z, ux, uy;
+};
+static __device__ __noinline__ RkState rk_substeps_move(double kappa, double s, int n, RkState in, double uz) {
+  double x = in.x, y = in.y, z = in.z, ux = in.ux, uy = in.uy;
   const double q0 = ux * ux + uy * uy;
   const double h = quot(s, (double)n);
   const double h6 = quot_by(h, 6.0, 1.0 / 6.0);
@@ -258,7 +261,19 @@ __device__ __forceinline__ void rk_move(double kappa, double s, int n, double& x
   z += uz * s;
   ux = U;
   uy = V;
+  return RkState{x, y, z, ux, uy};
 }
+// (called, not inlined: 14 KB of code that runs with the substep cap only)
+__device__ __forceinline__ void rk_move(double kappa, double s, int n, double& x, double& y, double& z, double& ux,
+                                        double& uy, double uz) {
+  const RkState r = rk_substeps_move(kappa, s, n, RkState{x, y, z, ux, uy}, uz);
+  x = r.x;
+  y = r.y;
+  z = r.z;
+  ux = r.ux;
+  uy = r.uy;
+}
+
 
 // Smallest turn angle t in [0, 2 pi) with sin(sigma t + beta) = d.
 __device__ __forceinline__ double first_turn(double d, double beta, double sigma) {
