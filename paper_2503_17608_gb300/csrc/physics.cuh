@@ -92,6 +92,22 @@ struct TrackRng {
     return w;
   }
   __device__ __forceinline__ double uniform() { return unit_from_bits(raw()); }
+  // Three draws: the block of the first and the next one.
+  __device__ __forceinline__ void raw3(unsigned long long& w1, unsigned long long& w2, unsigned long long& w3) {
+    const uint32_t block = ctr >> 1;
+    const bool odd = (ctr & 1u) != 0u;
+    uint4 a = cached;
+    if (block != cached_block) a = philox_block(make_uint4((uint32_t)tid, (uint32_t)(tid >> 32), block, 0u), key);
+    cached = philox_block(make_uint4((uint32_t)tid, (uint32_t)(tid >> 32), block + 1u, 0u), key);
+    cached_block = block + 1u;
+    ctr += 3u;
+    const unsigned long long alo = (unsigned long long)a.y << 32 | a.x, ahi = (unsigned long long)a.w << 32 | a.z;
+    const unsigned long long blo = (unsigned long long)cached.y << 32 | cached.x,
+                             bhi = (unsigned long long)cached.w << 32 | cached.z;
+    w1 = odd ? ahi : alo;
+    w2 = odd ? blo : ahi;
+    w3 = odd ? bhi : blo;
+  }
 };
 
 // Comparisons of doubles on their bit patterns (integer instructions instead
@@ -149,6 +165,16 @@ __device__ __forceinline__ double inverse_range(const double2* R, double r, doub
 // the same time whatever its active lanes, so the kinematics below take
 // reciprocal square roots once instead of a square root and divisions.
 
+// Near the poles: sin(theta) and sin(theta) / |u x x|, called (few directions
+// lie there).
+struct PoleFrame {
+  double sint, b;
+};
+static __device__ __noinline__ PoleFrame pole_frame(double t, double uy, double uz) {
+  const double sint = fast_sqrt(t);
+  return PoleFrame{sint, sint * fast_rsqrt(fma(uz, uz, uy * uy))};
+}
+
 // Rotate (ux, uy, uz) by polar cosine cost and azimuth 2 pi u_phi about
 // itself: frame e1 = (u x z)/|u x z|, e2 = u x e1 (e1 = x near the poles),
 // then renormalised. With n = |u x z|, q = n^2 and w = sin(theta)/n =
@@ -174,9 +200,9 @@ __device__ __forceinline__ void rotate_dir(double& ux, double& uy, double& uz, d
     vy = fma(C, uy, -A * ux);
     vz = fma(cost, uz, -B * q);
   } else {
-    const double sint = fast_sqrt(t);
-    const double B = sint * sp * fast_rsqrt(fma(uz, uz, uy * uy));
-    vx = fma(cost, ux, sint * cp);
+    const PoleFrame f = pole_frame(t, uy, uz);
+    const double B = f.b * sp;
+    vx = fma(cost, ux, f.sint * cp);
     vy = fma(cost, uy, B * uz);
     vz = fma(cost, uz, -B * uy);
   }
@@ -330,15 +356,21 @@ static __device__ __noinline__ double helix_side_distance(Curvature c, double x,
 // computed in FP64, by the same expressions as the plain FP64 sampler, so
 // the samples are bit-identical to it:
 //  * the FP32 quantities are evaluated from cancellation-free forms
-//    (1 - eps by expm1 or an algebraic rewrite, 2b - a likewise) with
+//    (1 - eps by e^x - 1 or an algebraic rewrite, 2b - a likewise) with
 //    relative errors below 2^-16 of the values the FP64 expressions
 //    approximate, and the FP64 expressions are within 2^-19 of them
 //    whenever 1 - eps >= 2^-30 and 2b - a >= 2^-30 (2k + 1) eps, which the
-//    filter checks;
+//    filter checks. The hardware's approximations suffice for that (ex2 2^-22,
+//    sqrt, rcp and the quotient 2^-21, documented): e^x from ex2(x log2 e) is
+//    within 2^-22 + |x| 2^-23 (below 2^-18.5 for |x| <= 15), e^x - 1 is taken
+//    from a five-term series below |x| = 1/8 (truncation 2^-24) and from e^x
+//    above (2^-19). They take a third of the instructions of the rounded
+//    library forms (sampler 10.6 -> 6.6 KB of code; asynchronous loop, 4 T
+//    calorimeter, 10,000 x 10 GeV 3.82 -> 3.50 ms, 100,000 27.6 -> 25.4 ms);
 //  * a decision is taken in FP32 only if the two sides differ by more than
 //    kFilterMargin = 2^-12 relative, far above both error bounds, so both
 //    evaluations take the same decision; otherwise (probability ~2^-11 per
-//    attempt) the FP64 test of the plain sampler decides.
+//    attempt) the FP64 test of the plain sampler decides, in a called function.
 // The filter covers k = E/m in [1e-4, 1e6] (Compton) and x = Tcut/T in
 // [1e-8, 1/2) (Moller); other inputs take the plain FP64 sampler.
 constexpr float kFilterMargin = 0x1p-12f;
@@ -362,6 +394,22 @@ __device__ __forceinline__ float f32_trunc(double v) {
   const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
   const unsigned e = ((hi >> 20) & 0x7FFu) - 1023u + 127u;
   return __uint_as_float((e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+}
+
+__device__ __forceinline__ float f32_exp(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.44269504f));
+  return r;
+}
+__device__ __forceinline__ float f32_expm1(float x) {
+  // x + x^2/2 + ... + x^5/120
+  const float q = fmaf(x, fmaf(x, fmaf(x, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f), 0.5f);
+  return fabsf(x) < 0.125f ? fmaf(x * x, q, x) : f32_exp(x) - 1.0f;
+}
+__device__ __forceinline__ float f32_sqrt(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // Klein-Nishina sampling of eps = E'/E by Butcher and Messel's
@@ -405,6 +453,20 @@ static __device__ __noinline__ double sample_compton_fp64(double E, TrackRng& rn
   return eps;
 }
 
+// The plain FP64 attempt of the filtered sampler below; the branch is decided
+// here if it is 0. Returns the branch if the attempt is accepted, else 0.
+static __device__ __noinline__ int compton_attempt_fp64(double k, double eps0sq, double a1, double w,
+                                                        unsigned long long w1, unsigned long long w2,
+                                                        unsigned long long w3, int branch, const double* mt) {
+  const double u2 = unit_from_bits(w2);
+  if (branch == 0) branch = (unit_from_bits(w1) * (a1 + 0.5 * w) < a1) ? 1 : 2;
+  const double e = branch == 1 ? fast_exp(-a1 * u2, mt) : fast_sqrt(fma(w, u2, eps0sq));
+  const double a = 1.0 - e;
+  const double b = k * e;
+  const double B = b * b * (1.0 + e * e);
+  return e * a * (2.0 * b - a) <= (1.0 - unit_from_bits(w3)) * B ? branch : 0;
+}
+
 // FP32-filtered Compton sampler (same draws, same results as
 // sample_compton_fp64). Per attempt, with u = u1..u3 and v = 1 - u:
 //  branch: u1 (a1 + a2) < a1;
@@ -417,8 +479,11 @@ static __device__ __noinline__ double sample_compton_fp64(double E, TrackRng& rn
 // The loop keeps only the accepted attempt's draw and branch; its FP64 value
 // is computed once after the loop, where the warp has reconverged (inside
 // the loop, lanes accepting at different attempts would each run it).
+// A caller that can come back gives a smaller attempt limit: ok is then
+// cleared with fewer than 3 kMaxAttempts draws taken, and sampling goes on
+// from the advanced draw counter.
 static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, double& cost, bool& ok,
-                                                     const double* mt) {
+                                                     const double* mt, int attempts = kMaxAttempts) {
   const double k = quot_by(E, kMe, 1.0 / kMe);
   // 1e-4 <= k <= 1e6 on the bits (negative and NaN k fall outside)
   if ((unsigned long long)(dbits(k) - dbits(1e-4)) > (unsigned long long)(dbits(1e6) - dbits(1e-4)))
@@ -434,9 +499,10 @@ static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, do
   unsigned long long w2_acc = 0;
   int branch_acc = 0;
   ok = false;
-  for (int attempt = 0; attempt < kMaxAttempts; ++attempt) {
+  for (int attempt = 0; attempt < attempts; ++attempt) {
     CELER_LANES(LS_COMPTON_TRY);
-    const unsigned long long w1 = rng.raw(), w2 = rng.raw(), w3 = rng.raw();
+    unsigned long long w1, w2, w3;
+    rng.raw3(w1, w2, w3);
     int branch = 0;   // 1 or 2 once decided
     int verdict = -1; // 1 accept, 0 reject, -1 undecided
     {
@@ -454,13 +520,13 @@ static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, do
         float ef, af, cf;
         if (branch == 1) {
           const float x = a1f * u2f;
-          ef = expf(-x);
-          af = -expm1f(-x);
-          cf = expm1f(a1f * v2f);
+          ef = f32_exp(-x);
+          af = -f32_expm1(-x);
+          cf = f32_expm1(a1f * v2f);
         } else {
-          ef = sqrtf(fmaf(wf, u2f, e0sqf));
-          af = wf * v2f / (1.0f + ef);
-          cf = k21f * wf * u2f / (ef + e0f);
+          ef = f32_sqrt(fmaf(wf, u2f, e0sqf));
+          af = __fdividef(wf * v2f, 1.0f + ef);
+          cf = __fdividef(k21f * wf * u2f, ef + e0f);
         }
         if (af >= kFilterTiny && cf >= kFilterTiny * k21f * ef) {
           const float bf = kf * ef;
@@ -475,14 +541,9 @@ static __device__ __noinline__ double sample_compton(double E, TrackRng& rng, do
       }
     }
     if (verdict == 0) continue;
-    if (verdict < 0) {  // the plain FP64 attempt
-      const double u2 = unit_from_bits(w2);
-      if (branch == 0) branch = (unit_from_bits(w1) * (a1 + 0.5 * w) < a1) ? 1 : 2;
-      const double e = branch == 1 ? fast_exp(-a1 * u2, mt) : fast_sqrt(fma(w, u2, eps0sq));
-      const double a = 1.0 - e;
-      const double b = k * e;
-      const double B = b * b * (1.0 + e * e);
-      if (!(e * a * (2.0 * b - a) <= (1.0 - unit_from_bits(w3)) * B)) continue;
+    if (verdict < 0) {
+      branch = compton_attempt_fp64(k, eps0sq, a1, w, w1, w2, w3, branch, mt);
+      if (branch == 0) continue;
     }
     w2_acc = w2;
     branch_acc = branch;
@@ -526,14 +587,26 @@ static __device__ __noinline__ double sample_moller_fp64(double T, double Tcut, 
   return eps;
 }
 
+// The plain FP64 attempt of the filtered sampler below.
+static __device__ __noinline__ bool moller_attempt_fp64(double T, double x, double y, unsigned long long w1,
+                                                        unsigned long long w2) {
+  const double g = quot_by(T, kMe, 1.0 / kMe) + 1.0;
+  const double g2 = g * g;
+  const double norm = quot(4.0, 9.0 * g2 - 10.0 * g + 5.0);
+  const double e = quot(x, fma(-unit_from_bits(w1), y, 1.0));
+  const double om = 1.0 - e;
+  const double eom = e * om;
+  const double fom2 = (g - 1.0) * (g - 1.0) * eom * eom - (2.0 * g2 + 2.0 * g - 1.0) * eom + g2;
+  return unit_from_bits(w2) * (om * om) <= norm * fom2;
+}
+
 // FP32-filtered Moller sampler (same draws, same results as
 // sample_moller_fp64). The proposal's denominator 1 - u1 (1 - 2x) is taken as
 // v1 + 2x u1 (no cancellation); the polynomial (g-1)^2 eom^2 - (2g^2 + 2g - 1)
 // eom + g^2 is at least 1/7 of the sum of its terms' magnitudes for g >= 1
 // and eom <= 1/4, and 9g^2 - 10g + 5 at least 1/6 of its terms', so their
 // FP32 relative errors stay below 2^-16; g - 1 = T/m is formed directly.
-// g, g^2 and the normalisation are needed in FP64 only for an undecided
-// attempt; the accepted attempt's eps is computed once, after the loop.
+// The accepted attempt's eps is computed once, after the loop.
 static __device__ __noinline__ double sample_moller(double T, double Tcut, TrackRng& rng, bool& ok) {
   const double x = quot(Tcut, T);
   // 1e-8 <= x < 1/2 on the bits (negative and NaN x fall outside)
@@ -543,13 +616,11 @@ static __device__ __noinline__ double sample_moller(double T, double Tcut, Track
   const float tmf = f32_trunc(T) * (float)(1.0 / kMe);  // g - 1
   const float gf = tmf + 1.0f;
   const float g2f = gf * gf;
-  const float normf = 4.0f / fmaf(9.0f, g2f, fmaf(-10.0f, gf, 5.0f));
+  const float normf = __fdividef(4.0f, fmaf(9.0f, g2f, fmaf(-10.0f, gf, 5.0f)));
   const float c1f = tmf * tmf;
   const float c2f = fmaf(2.0f, g2f, fmaf(2.0f, gf, -1.0f));
   const float xf = f32_trunc(x);
   const float txf = 2.0f * xf;
-  double g = 0.0, g2 = 0.0, norm = 0.0;
-  bool fp64_ready = false;
   unsigned long long w1_acc = 0;
   ok = false;
   for (int attempt = 0; attempt < kMaxAttempts; ++attempt) {
@@ -560,7 +631,7 @@ static __device__ __noinline__ double sample_moller(double T, double Tcut, Track
       const unsigned long long n1 = draw_numerator(w1);
       const float u1f = f32_scaled_2m53(n1), v1f = f32_scaled_2m53(k2p53 - n1);
       const float u2f = f32_scaled_2m53(draw_numerator(w2));
-      const float ef = xf / fmaf(u1f, txf, v1f);
+      const float ef = __fdividef(xf, fmaf(u1f, txf, v1f));
       const float omf = 1.0f - ef;
       const float eomf = ef * omf;
       const float L = u2f * (omf * omf);
@@ -572,19 +643,7 @@ static __device__ __noinline__ double sample_moller(double T, double Tcut, Track
       }
     }
     if (verdict == 0) continue;
-    if (verdict < 0) {  // the plain FP64 attempt
-      if (!fp64_ready) {
-        g = quot_by(T, kMe, 1.0 / kMe) + 1.0;
-        g2 = g * g;
-        norm = quot(4.0, 9.0 * g2 - 10.0 * g + 5.0);
-        fp64_ready = true;
-      }
-      const double e = quot(x, fma(-unit_from_bits(w1), y, 1.0));
-      const double om = 1.0 - e;
-      const double eom = e * om;
-      const double fom2 = (g - 1.0) * (g - 1.0) * eom * eom - (2.0 * g2 + 2.0 * g - 1.0) * eom + g2;
-      if (!(unit_from_bits(w2) * (om * om) <= norm * fom2)) continue;
-    }
+    if (verdict < 0 && !moller_attempt_fp64(T, x, y, w1, w2)) continue;
     w1_acc = w1;
     ok = true;
     break;
