@@ -343,16 +343,17 @@ celer_status celer_set_parent_reuse(celer_ctx* ctx, int on);
 /* Scheduling of the asynchronous loop (CELER_LOOP_ASYNC) for the block-local
  * policy. on = 0: block passes, as in the synchronous loops. on = 1: every
  * warp runs its own loop. It takes up to 32 tracks waiting for the same kind
- * of step (particle type and next action) from its block's queues in shared
- * memory, steps them, and queues the survivors again by their next kind. A
- * track then moves on as soon as its own step is done instead of waiting for
- * its block's slowest group. Charged tracks are taken before photons (their
- * steps form a shower's longest chains), and in runs without an iteration
- * budget all but the first two warps of a block take only full pieces of 32
- * (budgeted runs, such as a serving loop's chunks, let every warp take any
- * piece). A block holds at most 1024 live tracks in this
- * mode; a block that starts a run with more runs block passes. Histories do
- * not change. On by default. Takes effect at the next run. on outside
+ * of work (photon flight, electron steps, or one interaction) from its
+ * block's queues in shared memory, moves them by one or more steps, and
+ * queues the survivors again by their next kind. A track then moves on as
+ * soon as its own step is done instead of waiting for its block's slowest
+ * group. Charged tracks are taken before photons (their steps form a shower's
+ * longest chains), and in runs without an iteration budget all but the first
+ * two warps of a block take only full pieces of 32 (budgeted runs, such as a
+ * serving loop's chunks, let every warp take any piece). A block keeps its
+ * live tracks in shared memory, at most 1024 of them (256 with more than four
+ * materials); a block that starts a run with more steps them in turns.
+ * Histories do not change. On by default. Takes effect at the next run. on outside
  * {0, 1}: CELER_ERR_INVALID. */
 celer_status celer_set_async_warps(celer_ctx* ctx, int on);
 
@@ -496,20 +497,19 @@ celer_status celer_debug_partition(celer_ctx* ctx, uint8_t* keys_out, uint32_t* 
  * host_out receives three values: warp-level visits, the lanes active at
  * them summed (mean active lanes = lanes / visits), and the SM cycles spent
  * there summed where the site is timed (0 elsewhere). Sites: 0-7 the
- * per-warp pieces of the asynchronous loop by key (particle type and next
- * action, in the order photon boundary, electron boundary, electron range,
- * Compton, photoelectric, pair, Moller, brems; lanes = tracks claimed;
- * timed from the claim to the survivors' requeue), 8 its fills (timed), 9
+ * per-warp pieces of the asynchronous loop by key (in the order photon
+ * flights, electron steps, 2 unused, Compton, 4 unused, pair, Moller, brems;
+ * lanes = tracks claimed; timed from the claim to the survivors' requeue), 8
+ * its fills (timed), 9
  * the step limit, 10 the along-step, 11-15 the Compton, photoelectric, pair,
  * Moller and brems interactions, 16 and 17 one rejection attempt of the
  * Compton and Moller samplers, 18 the side-plane distance along the helix,
  * 19 the per-warp loop's rounds that found nothing to do (timed), 20-22 the
- * photon crossing pieces timed in three parts (choice and claim, the step,
- * the next step limit and requeue), 23-25 the same for electron crossings,
- * 26-30 a photon's step limit timed in five parts (state loads, grid position,
- * cross sections, distances to the planes, the rest with the stores), 31 the
- * per-warp loop's queueing of a track by its next kind, 32-34 the Compton
- * pieces timed in three parts as the crossings.
+ * photon flight pieces timed in three parts (choice and claim, the steps, the
+ * requeue), 23-25 the same for the electron pieces, 26-30 a photon's step
+ * limit in the other loops timed in five parts (state loads, grid position,
+ * cross sections, distances to the planes, the rest with the stores), 31
+ * unused, 32-34 the Compton pieces timed in three parts as the flights.
  * The counters cover every kernel launched since the last read on the
  * current device and are cleared by the read. *n_out receives the sites
  * written. Null pointers or n_max < 0: CELER_ERR_INVALID. */

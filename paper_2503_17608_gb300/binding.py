@@ -505,11 +505,11 @@ def debug_fp64_rate(blocks_per_sm: int = 4, iters: int = 40000):
 LANE_SITES = ["piece g_geom", "piece e_geom", "piece e_range", "piece compton", "piece pe", "piece pair",
               "piece moller", "piece brems", "fill", "step_limit", "along", "compton", "photoelectric", "pair",
               "moller", "brems", "compton_attempt", "moller_attempt", "helix_side", "idle",
-              "photon_crossing: claim", "photon_crossing: step", "photon_crossing: next limit",
-              "electron_crossing: claim", "electron_crossing: step", "electron_crossing: next limit",
+              "photon flight: claim", "photon flight: steps", "photon flight: requeue",
+              "electron steps: claim", "electron steps: steps", "electron steps: requeue",
               "photon limit: loads", "photon limit: grid (log)", "photon limit: cross sections",
-              "photon limit: planes", "photon limit: rest and stores", "queue push",
-              "compton: claim", "compton: step", "compton: next limit"]
+              "photon limit: planes", "photon limit: rest and stores", "unused",
+              "compton: claim", "compton: step", "compton: requeue"]
 
 
 def debug_lane_counts():

@@ -21,7 +21,8 @@ LIB = os.path.join(HERE, "libceler_gb.so")
 LANES_BUILD = os.path.join(HERE, "_build_lanes")
 LANES_LIB = os.path.join(HERE, "libceler_gb_lanes.so")
 SOURCES = ["step.cu", "tables.cu", "driver.cu", "debug.cu", "noalloc.cu", "serve.cu"]
-HEADERS = ["common.cuh", "physics.cuh", "fastmath.cuh", "launch.h", "tables.h", "block_pass.cuh", "async_loop.cuh"]
+HEADERS = ["common.cuh", "physics.cuh", "fastmath.cuh", "launch.h", "tables.h", "block_pass.cuh", "async_loop.cuh",
+           "warp_loop.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

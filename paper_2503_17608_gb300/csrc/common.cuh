@@ -195,6 +195,7 @@ struct Params {
   int n_layers;
   int n_materials;
   const double* zb;        // n_layers + 1
+  uint32_t static_bytes;   // tables, layer planes and materials in shared memory (a multiple of 16)
   const int32_t* layer_mat;
   double hx, hy, Bz;
   double field_bk, field_inv_bk;  // Bz times the curvature constant, and its inverse (0 without field)
@@ -233,7 +234,8 @@ struct Params {
 // copies by block to keep the atomics apart. The product build compiles every
 // site to nothing.
 enum LaneSite : int {
-  LS_PIECE = 0,        // + K_* key: per-warp pieces of the asynchronous loop (tracks claimed)
+  LS_PIECE = 0,        // + K_* key: per-warp pieces of the asynchronous loop (tracks claimed; photon
+                       // flights under K_G_GEOM, electron steps under K_E_GEOM)
   LS_FILL = 8,         // per-warp fills of the asynchronous loop (initializers taken)
   LS_STEP_LIMIT = 9,   // step limit of a live track
   LS_ALONG = 10,       // along-step
@@ -242,14 +244,13 @@ enum LaneSite : int {
   LS_MOLLER_TRY = 17,  // one rejection attempt of the Moller sampler
   LS_HELIX_SIDE = 18,  // side-plane distance along the helix
   LS_IDLE = 19,        // per-warp loop rounds of the asynchronous loop that found nothing to do
-  LS_T_PHOTON = 20,    // photon crossing pieces timed in three parts: choice and claim, the
-                       // step, the next step limit and requeue (20, 21, 22)
-  LS_T_ELECTRON = 23,  // the same for electron crossing pieces (23, 24, 25)
+  LS_T_PHOTON = 20,    // photon flight pieces timed in three parts: choice and claim, the
+                       // steps, the requeue (20, 21, 22)
+  LS_T_ELECTRON = 23,  // the same for the electron pieces (23, 24, 25)
   LS_T_LIMIT = 26,     // the step limit of a photon timed in five parts: the state loads, the
                        // grid position (logarithm), the cross sections, the distances to the
                        // planes, the rest with the stores (26-30)
-  LS_T_PUSH = 31,      // queueing a track by its next kind (per-warp loop)
-  LS_T_COMPTON = 32,   // Compton pieces timed in three parts as the crossings (32, 33, 34)
+  LS_T_COMPTON = 32,   // Compton pieces timed in three parts as the flights (32, 33, 34)
   kLaneSites = 35
 };
 constexpr int kLaneCopies = 16;

@@ -444,6 +444,7 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
   p.n_keys = keys_of(p.policy);
   p.n_layers = L;
   p.n_materials = pb->n_materials;
+  p.static_bytes = (uint32_t)static_smem_bytes(p.n_materials, L);
   p.hx = pb->half_x;
   p.hy = pb->half_y;
   p.Bz = pb->Bz;

@@ -13,6 +13,13 @@ struct StagedPrimary {
   int32_t layer, ptype;
 };
 
+// Bytes of the static tables in shared memory (carve_static), in 16s.
+inline size_t static_smem_bytes(int n_materials, int n_layers) {
+  const size_t n = (size_t)n_materials * kCols * kGrid * sizeof(double2) + (size_t)(n_layers + 1) * sizeof(double) +
+                   (size_t)n_layers * sizeof(int32_t);
+  return (n + 15) & ~(size_t)15;
+}
+
 struct LaunchShape {
   int tile_grid;       // persistent grid of the tile kernels (fill, step limit, scatter)
   int step_grid;       // persistent grid of the phase-merged step kernel
@@ -21,6 +28,8 @@ struct LaunchShape {
   int loop_grid;       // co-resident grid of the persistent loop kernel
   int block;           // threads per block of the step / along-step / interaction kernels
   size_t static_smem;  // tables + layer planes + layer materials in shared memory
+  size_t warp_smem;    // the per-warp schedule: the block's tracks beside them
+  bool warp_small;     // its variant with fewer tracks per block
 };
 
 cudaError_t configure_kernels(const Params& p, int block, LaunchShape* shape);
@@ -48,7 +57,8 @@ void launch_begin_run(const Params& p, unsigned long long budget, cudaStream_t s
 // persistent loop
 cudaError_t launch_loop(const Params& p, const LaunchShape& sh, cudaStream_t s);
 // Asynchronous block loop (block-pass policies): the buffer entries' states,
-// then one cooperative launch; p.ring_state must be set.
+// then one cooperative launch (per-warp schedule or block passes);
+// p.ring_state must be set.
 void launch_async_prepare(const Params& p, cudaStream_t s);
 // Check of the asynchronous loop's queue waits (k_queue_wait_probe).
 cudaError_t launch_queue_wait_probe(const Params& p, int which, long long timeout, cudaStream_t s);

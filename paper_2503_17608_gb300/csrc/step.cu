@@ -24,10 +24,12 @@ __device__ __forceinline__ uint32_t row_of(const Params& p, uint32_t ev) {
   return ev < p.max_events ? ev : row_modulo(ev, p.max_events);
 }
 
+static __device__ __noinline__ int z_bin(double z, double z0, double zscale, int n_bins) {
+  int b = __double2int_rd((z - z0) * zscale);  // (int)floor, one conversion
+  return b < 0 ? 0 : (b > n_bins - 1 ? n_bins - 1 : b);
+}
 __device__ __forceinline__ int tally_bin(const Params& p, int layer, double z) {
-  if (p.tally_mode == 1) return layer;
-  int b = __double2int_rd((z - p.z0) * p.zscale);  // (int)floor, one conversion
-  return b < 0 ? 0 : (b > p.n_bins - 1 ? p.n_bins - 1 : b);
+  return p.tally_mode == 1 ? layer : z_bin(z, p.z0, p.zscale, p.n_bins);
 }
 
 __device__ __forceinline__ void deposit(const Params& p, uint32_t ev, uint32_t prim, int layer, double z, double e) {
@@ -92,10 +94,7 @@ __device__ __forceinline__ unsigned ring_lap_code(const Params& p, unsigned long
 // Bounded wait of one thread for entry `index` to reach state `code`. After
 // `timeout` cycles (~1 s by default), or if another wait gave up first (abort
 // word), it sets the abort word and ERR_BARRIER_TIMEOUT and returns false.
-__device__ __noinline__ bool ring_wait(const Params& p, unsigned long long index, unsigned code,
-                                       long long timeout = kBarrierTimeoutCycles) {
-  const unsigned* st = p.ring_state + (index & p.ring_mask);
-  if (ld_acquire_u32(st) == code) return true;
+__device__ __noinline__ bool ring_wait_poll(const Params& p, const unsigned* st, unsigned code, long long timeout) {
   unsigned* abort_word = p.barrier + 2;
   const long long t0 = clock64();
   for (;;) {
@@ -108,6 +107,11 @@ __device__ __noinline__ bool ring_wait(const Params& p, unsigned long long index
       return false;
     }
   }
+}
+__device__ __forceinline__ bool ring_wait(const Params& p, unsigned long long index, unsigned code,
+                                          long long timeout = kBarrierTimeoutCycles) {
+  const unsigned* st = p.ring_state + (index & p.ring_mask);
+  return ld_acquire_u32(st) == code || ring_wait_poll(p, st, code, timeout);
 }
 
 // An initializer record by its 16-byte parts.
@@ -1673,6 +1677,7 @@ __global__ void __launch_bounds__(kTile, 1) k_loop_local(Params p) {
 }
 
 #include "async_loop.cuh"
+#include "warp_loop.cuh"
 
 // Check of the bounded waits: every block but `absent` meets at a grid
 // barrier that `absent` never reaches, so the waiters must give up after
@@ -1781,8 +1786,7 @@ cudaError_t configure_kernels(const Params& p, int block, LaunchShape* sh) {
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const size_t stat = (size_t)p.n_materials * kCols * kGrid * sizeof(double2) +
-                      (size_t)(p.n_layers + 1) * sizeof(double) + (size_t)p.n_layers * sizeof(int32_t);
+  const size_t stat = static_smem_bytes(p.n_materials, p.n_layers);
   sh->static_smem = stat;
   sh->block = block;
   const void* with_smem[] = {(const void*)k_fill_step, (const void*)k_step, (const void*)k_fill,
@@ -1792,6 +1796,19 @@ cudaError_t configure_kernels(const Params& p, int block, LaunchShape* sh) {
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stat);
     if (e != cudaSuccess) return e;
   }
+  // the per-warp schedule keeps a block's tracks in shared memory: as many as
+  // fit beside the static tables (1,024 up to four materials, else 256)
+  int max_smem = 0;
+  e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  cudaFuncAttributes fa{};
+  e = cudaFuncGetAttributes(&fa, (const void*)k_loop_warps<kWarpTracks>);
+  if (e != cudaSuccess) return e;
+  sh->warp_small = fa.sharedSizeBytes + TrackCache<kWarpTracks>::kBytes + stat + (size_t)p.n_layers * sizeof(double) > (size_t)max_smem;
+  sh->warp_smem = stat + (size_t)p.n_layers * sizeof(double) + (sh->warp_small ? TrackCache<kWarpTracksSmall>::kBytes : TrackCache<kWarpTracks>::kBytes);
+  const void* warps = sh->warp_small ? (const void*)k_loop_warps<kWarpTracksSmall> : (const void*)k_loop_warps<kWarpTracks>;
+  e = cudaFuncSetAttribute(warps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh->warp_smem);
+  if (e != cudaSuccess) return e;
   sh->tile_grid = occupancy_grid((const void*)k_fill_step, kTile, stat, sms, (int)p.n_tiles);
   const int cap_action = (int)((p.n_slots + block - 1) / block);
   sh->step_grid = occupancy_grid((const void*)k_step, block, stat, sms, cap_action);
@@ -1808,6 +1825,10 @@ cudaError_t configure_kernels(const Params& p, int block, LaunchShape* sh) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb_async, (const void*)k_loop_async, kTile, stat);
   if (e != cudaSuccess) return e;
   if (nb_async < nb) nb = nb_async;
+  int nb_warps = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb_warps, warps, kWarpThreads, sh->warp_smem);
+  if (e != cudaSuccess) return e;
+  if (nb_warps < nb) nb = nb_warps;
   sh->loop_grid = (nb < 1 ? 1 : nb) * sms;
   if (sh->loop_grid > kMaxLoopBlocks) sh->loop_grid = kMaxLoopBlocks;  // size of the per-block arrays
   return cudaGetLastError();
@@ -1858,6 +1879,10 @@ void launch_begin_run(const Params& p, unsigned long long budget, cudaStream_t s
 void launch_async_prepare(const Params& p, cudaStream_t s) { k_async_prepare<<<256, 256, 0, s>>>(p); }
 cudaError_t launch_loop_async(const Params& p, const LaunchShape& sh, cudaStream_t s) {
   void* args[] = {const_cast<Params*>(&p)};
+  if (p.policy == POLICY_LOCAL && p.async_warps) {
+    const void* fn = sh.warp_small ? (const void*)k_loop_warps<kWarpTracksSmall> : (const void*)k_loop_warps<kWarpTracks>;
+    return cudaLaunchCooperativeKernel(fn, dim3(sh.loop_grid), dim3(kWarpThreads), args, sh.warp_smem, s);
+  }
   return cudaLaunchCooperativeKernel((const void*)k_loop_async, dim3(sh.loop_grid), dim3(kTile), args, sh.static_smem,
                                      s);
 }
