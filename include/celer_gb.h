@@ -391,7 +391,7 @@ celer_status celer_kernel_timing(celer_ctx* ctx, const char** names, double* tot
  * is pending on the calling thread, the call launches nothing, leaves that
  * error pending and returns CELER_ERR_CUDA.
  *
- * Working memory is one fixed array inside the library (256 KiB per device
+ * Working memory is one fixed array inside the library (16 KiB per device
  * that loads it, held until the process exits): n <= 2^20, n_keys <= 16,
  * otherwise CELER_ERR_INVALID. Every call on a device shares that array, so
  * calls whose work overlaps on the GPU (other streams, other host threads)
