@@ -1,9 +1,8 @@
 // The asynchronous step loop (CELER_LOOP_ASYNC) of the block-pass policies:
 // the persistent kernel in which every block runs its own passes with no
-// grid barrier (k_loop_async), the per-warp schedule of the block-local
-// policy (warp_queue_loop and its shared-memory queues), the start-of-run
-// kernel that sets the buffer entries' states (k_async_prepare), and the
-// check of the bounded queue waits (k_queue_wait_probe). Included by step.cu
+// grid barrier (k_loop_async), the kernel that sets the buffer entries' states
+// (k_async_prepare), and the waits and accesses of the per-warp schedule's
+// queues (warp_loop.cuh) with their check (k_queue_wait_probe). Included by step.cu
 // inside its anonymous namespace, after the block passes (local_pass,
 // data_pass) and the buffer protocol (ring_wait, take_initializer) it uses.
 #pragma once
@@ -26,11 +25,14 @@ __device__ PassCounts block_total(const PassCounts& n) {
   return out;
 }
 
-// Start of an asynchronous run: the buffer entries' states from head and
-// tail (entries in [head, tail) written and unread, the others free for
-// their next writer) and the count of ended tracks, head - alive (every
-// track came from a buffer entry; a pair photon that reuses its parent's
-// slot continues the parent's count).
+// The buffer entries' states from head and tail (entries in [head, tail)
+// written and unread, the others free for their next writer) and the count of
+// ended tracks, head - alive (every track came from a buffer entry; a pair
+// photon that reuses its parent's slot continues the parent's count). An
+// asynchronous run leaves all of it as the next one needs it, and so do the
+// kernels that queue primaries; only after iterations of the synchronous
+// loops, which keep neither, or an error is it made anew (32 MB of states at
+// 2^20 slots, 10 us).
 __global__ void k_async_prepare(Params p) {
   const unsigned long long head = p.ctl->head, tail = p.ctl->tail;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -43,6 +45,7 @@ __global__ void k_async_prepare(Params p) {
     p.ctl->finished = head - p.ctl->alive;
     p.ctl->avail = tail - head;
     p.ctl->async_passes = 0;
+    p.ctl->vacant_seen = 0;
     p.ctl->done_x = 0u;
   }
 }
@@ -97,8 +100,12 @@ __device__ __forceinline__ void end_async_block(const Params& p, int nb, unsigne
     __threadfence();
     c->iteration = __ldcg(&c->iteration) + __ldcg(&c->async_passes);
     const unsigned long long queued = __ldcg(&c->tail) - __ldcg(&c->head), alive = __ldcg(&c->alive);
+    // (the per-warp schedule's blocks count their vacant slots themselves)
+    if (p.run_budget != 0ull && __ldcg(&c->vacant_seen) != c->total_vacant) atomicOr(&c->error, ERR_VACANCY);
+    c->vacant_seen = 0;
     c->total_vacant = (unsigned long long)p.n_slots - alive;
     c->cont = (alive + queued > 0 && __ldcg(&c->error) == 0u) ? 1u : 0u;
+    c->async_passes = 0;
     c->done_x = 0u;
   }
 }

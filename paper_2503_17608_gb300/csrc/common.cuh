@@ -155,7 +155,12 @@ struct Ctl {
   unsigned long long finished;
   unsigned long long avail;          // written entries not yet claimed by a reader (may dip below 0 briefly)
   unsigned long long async_passes;
+  unsigned long long vacant_seen;    // vacant slots the blocks of a per-warp run counted at its start
   unsigned int done_x;
+  // primaries in device memory: a record of the batch was rejected, and the
+  // last-block ticket of the push
+  unsigned int push_bad;
+  unsigned int done_push;
 };
 
 struct TraceRow {
@@ -205,6 +210,7 @@ struct Params {
   int reuse_parent;        // 1: a pair's first photon starts in the parent's slot (Sec. 3.2)
   int field_cap;           // 0: exact helix; > 0: Runge-Kutta substeps, at most this many per step
   int async_warps;         // asynchronous loop, block-local policy: 1 per-warp scheduling, 0 block passes
+  unsigned long long run_budget;  // per-warp schedule: pieces of the run (~0: no limit), set in its Params
   const double2* tables;   // [mat][col][kGrid] (value, next - value)
   const double* mtab;      // log/exp reduction tables (fastmath.cuh)
   double lnEmin, inv_dl, dl;

@@ -63,7 +63,12 @@ void launch_async_prepare(const Params& p, cudaStream_t s);
 // Check of the asynchronous loop's queue waits (k_queue_wait_probe).
 cudaError_t launch_queue_wait_probe(const Params& p, int which, long long timeout, cudaStream_t s);
 cudaError_t launch_loop_async(const Params& p, const LaunchShape& sh, cudaStream_t s);
-void launch_push_primaries(const Params& p, const StagedPrimary* d_prim, uint32_t n, cudaStream_t s);
+void launch_push_primaries(const Params& p, const StagedPrimary* prim, uint32_t n, unsigned long long base,
+                           uint32_t* states, cudaStream_t s);
+void launch_reset_event(double* tally, int n_bins, double* escaped, unsigned* event_live, cudaStream_t s);
+// Up to two runs of 32-bit words into pinned host memory, in one launch.
+void launch_copy_out(void* dst, const void* src, uint32_t words, void* dst2, const void* src2, uint32_t words2,
+                     cudaStream_t s);
 
 // Primary record as laid out by the C ABI (celer_primary).
 struct DevicePrimary {
@@ -73,7 +78,7 @@ struct DevicePrimary {
   int32_t ptype, pad;
 };
 void launch_push_device_primaries(const Params& p, const DevicePrimary* src, uint32_t n, uint32_t event,
-                                  unsigned long long tid0, uint32_t prim0, cudaStream_t s);
+                                  unsigned long long tid0, uint32_t prim0, uint32_t* states, cudaStream_t s);
 
 // Active-lane counters of the instrumented build (-DCELER_LANE_COUNTERS):
 // 3 x n_sites values (visits, lanes, cycles) summed over the copies, then

@@ -864,6 +864,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   const SharedStatic ss = carve_static(p, smem_raw + TrackCache<kCap>::kBytes);
   __shared__ unsigned s_head[kWarpKinds + 1], s_tail[kWarpKinds + 1];
   __shared__ unsigned s_live, s_filling, s_exit, s_drain, s_parked, s_cursor, s_kind, s_looked, s_deferred;
+  __shared__ unsigned s_vacant;
   __shared__ unsigned long long s_pieces;
   const int nb = (int)gridDim.x, bid = (int)blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -873,11 +874,17 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   const uint32_t n_own = (uint32_t)bid < p.n_chunks ? (p.n_chunks - (uint32_t)bid + nb - 1) / nb : 0u;
   const bool owns_last = n_own > 0 && (uint32_t)bid + (uint32_t)nb * (n_own - 1u) == p.n_chunks - 1u;
   const unsigned owned = n_own * 32u - (owns_last ? p.n_chunks * 32u - p.n_slots : 0u);
-  const unsigned live0 = owned - __ldcg(&p.block_vacant[bid]);
   const unsigned n_entries = owned < (unsigned)kCap ? owned : (unsigned)kCap;
   const unsigned long long max_pieces = __ldcg(&ctl->max_iterations);  // per run
-  const unsigned long long budget_end = __ldcg(&ctl->budget_end);
-  const unsigned long long budget = budget_end == ~0ull ? ~0ull : budget_end - __ldcg(&ctl->iteration);
+  const unsigned long long budget = p.run_budget;
+  if (threadIdx.x == 0) s_vacant = 0u;
+  __syncthreads();
+  {  // the block's vacant slots
+    unsigned v = 0;
+    for (uint32_t m = threadIdx.x; m < n_own; m += blockDim.x) v += __ldcg(&p.vacant[(uint32_t)bid + (uint32_t)nb * m]);
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0 && v) atomicAdd(&s_vacant, v);
+  }
   for (unsigned c = threadIdx.x; c < (unsigned)kCap; c += blockDim.x) {
     tc.meta(c) = 0u;
     for (int k = 0; k < kWarpKinds; ++k) *tc.queue(k, c) = 0u;
@@ -891,23 +898,23 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     s_live = 0u;
     s_filling = 0u;
     s_exit = 0u;
-    s_drain = budget == 0ull ? 1u : 0u;
+    s_drain = 0u;
     s_pieces = 0ull;
-    s_parked = live0;  // every live track waits in its slot until an entry takes it
     s_cursor = 0u;
+    s_parked = 0u;
     s_kind = (unsigned)W_PHOTON;
     s_deferred = 0u;
     s_looked = (unsigned)clock64() - 2u * kLookCycles;
-    if (__ldcg(&ctl->local_blocks) != (unsigned)nb) {  // vacancy counts made for another grid
-      atomicOr(&ctl->error, ERR_VACANCY);
-      atomicExch(abort_word, 1u);
-      s_exit = 1u;
-    }
   }
   double* thick = reinterpret_cast<double*>(smem_raw + TrackCache<kCap>::kBytes + p.static_bytes);  // layer thicknesses
   for (int l = threadIdx.x; l < p.n_layers; l += blockDim.x) thick[l] = p.zb[l + 1] - p.zb[l];
   stage_static(p, ss);  // ends with a block barrier
-  if (live0 > 0 && live0 <= n_entries && s_exit == 0u && s_drain == 0u) {
+  const unsigned live0 = owned - s_vacant;
+  if (threadIdx.x == 0) {
+    atomicAdd(&ctl->vacant_seen, (unsigned long long)s_vacant);
+    if (live0 > n_entries) s_parked = live0;  // they wait in their slots until entries take them
+  }
+  if (live0 > 0 && live0 <= n_entries) {
     // the live tracks of the block's chunks, one chunk per warp at a time,
     // take the first entries
     for (uint32_t m = (uint32_t)warp; m < n_own; m += blockDim.x >> 5) {
@@ -931,10 +938,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
         todo &= ~m2;
       }
     }
-    if (threadIdx.x == 0) {
-      s_live = live0;
-      s_parked = 0u;
-    }
+    if (threadIdx.x == 0) s_live = live0;
   }
   __syncthreads();
   unsigned steps = 0, killed = 0, fill = 0, events = 0;
@@ -1243,8 +1247,5 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   const unsigned live = s_live;
   if (live > 0)
     store_tracks(p, tc, reinterpret_cast<uint16_t*>(const_cast<unsigned*>(tc.queue(0, 0u))), n_entries, bid, nb);
-  if (threadIdx.x == 0) {
-    p.block_vacant[bid] = owned - live - s_parked;
-    end_async_block(p, nb, s_pieces);
-  }
+  if (threadIdx.x == 0) end_async_block(p, nb, s_pieces);
 }

@@ -73,3 +73,37 @@ def test_event_ids_beyond_the_tally_rows():
     for e in (1000, 7001):
         want = o["edep"][prim["event"] == e].sum(0)
         np.testing.assert_allclose(g["tally"][e][0], want, rtol=0, atol=1e-9 * want.max())
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 4097])
+def test_queued_primaries_between_runs_of_all_loops(n):
+    """Runs of the asynchronous loop take up the buffer as the last run and the
+    pushes since left it; synchronous runs in between make them set it up
+    anew. Host batches below and above the size read in place, device batches,
+    and a budgeted run in the middle."""
+    import torch
+
+    # (room for two batches: a budgeted run leaves most of its own queued)
+    prob = wl.water_cube_problem(n_slots=2048, init_capacity=16384, history_capacity=8 * n, sort_policy=wl.SORT_LOCAL)
+    runs = [(wl.SORT_LOCAL, binding.LOOP_ASYNC, 0), (wl.SORT_LOCAL, binding.LOOP_ASYNC, 2),
+            (wl.SORT_DATA, binding.LOOP_ASYNC, 0), (wl.SORT_LOCAL, binding.LOOP_ASYNC, 0),
+            (wl.SORT_NONE, binding.LOOP_PERSISTENT, 3), (wl.SORT_LOCAL, binding.LOOP_ASYNC, 0)]
+    prim = wl.water_cube_primaries(n)
+    dev = torch.from_numpy(binding.to_c_primaries(prim).view(np.uint8).copy()).cuda()
+    with binding.Context(prob) as ctx:
+        for k, (policy, mode, budget) in enumerate(runs):
+            ctx.set_sort_policy(policy)
+            if k % 2:
+                ctx.add_primaries_device(k, dev.data_ptr(), n)
+            else:
+                prim["event"][:] = k
+                ctx.add_primaries(k, prim)
+            ctx.run_iterations(mode, budget=budget)
+        s = ctx.stats()
+        assert s["alive"] == 0 and s["queued"] == 0
+        hist, edep = ctx.read_history(0, len(runs) * n)
+    for k in range(len(runs)):
+        prim["event"][:] = k
+        o = run_oracle(prob, prim)
+        np.testing.assert_array_equal(hist["steps"][k * n:(k + 1) * n], o["hist"]["steps"])
+        np.testing.assert_allclose(edep[k * n:(k + 1) * n], o["edep"], rtol=1e-9, atol=1e-9 * 10.0)
