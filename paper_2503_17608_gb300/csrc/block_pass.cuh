@@ -61,7 +61,8 @@ __device__ __forceinline__ void count_block_vacancies(const Params& p, int bid, 
 // thus spread over all SMs (a block fills its lowest vacancies, in its chunk
 // order), and the fill stays deterministic. s_v holds v_b; vmin and vmax
 // are their extremes. When every block has room for take/nb + 1 the level
-// is take/nb; otherwise one warp finds it by bisection. A block takes at most
+// is take/nb, and the quotas follow from it without a scan; otherwise one warp
+// finds it by bisection. A block takes at most
 // `cap` (its counts and the take are clamped); returns the take planned,
 // which the caller stores as the next fill_take.
 __device__ unsigned long long plan_block_quotas(const Params& p, uint32_t* s_v, int nb, unsigned vmin, unsigned vmax,
@@ -85,12 +86,15 @@ __device__ unsigned long long plan_block_quotas(const Params& p, uint32_t* s_v, 
     vmax = cap;
   }
   const unsigned long long l0 = take / (unsigned)nb;
-  if (l0 + 1 <= vmin) {
+  if (l0 + 1 <= vmin) {  // every block works its quota out itself (load_block_iter)
     if (threadIdx.x == 0) {
-      s_level = (unsigned)l0;
-      s_extra = (unsigned)(take - l0 * (unsigned)nb);
+      p.ctl->quota_level = (unsigned)l0;
+      p.ctl->quota_extra = (unsigned)(take - l0 * (unsigned)nb);
     }
-  } else if (threadIdx.x < 32) {
+    return take;
+  }
+  if (threadIdx.x == 0) p.ctl->quota_level = 0xFFFFFFFFu;
+  if (threadIdx.x < 32) {
     unsigned lo = 0, hi = vmax;  // S(0) = 0 <= take <= S(vmax) = sum v_b
     unsigned long long s_lo = 0;
     while (lo < hi) {
@@ -213,6 +217,11 @@ __device__ __forceinline__ BlockIter load_block_iter(const Params& p, int bid, i
   it.blocks_ok = __ldcg(&c->local_blocks) == (unsigned)nb;
   it.quota = __ldcg(&p.block_quota[bid]);
   it.prefix = __ldcg(&p.block_prefix[bid]);
+  const unsigned level = __ldcg(&c->quota_level), extra = __ldcg(&c->quota_extra);
+  if (level != 0xFFFFFFFFu) {
+    it.quota = level + ((unsigned)bid < extra ? 1u : 0u);
+    it.prefix = (unsigned long long)level * (unsigned)bid + min((unsigned)bid, extra);
+  }
   it.vtot = __ldcg(&p.block_vacant[bid]);
   const uint32_t n_own = (uint32_t)bid < p.n_chunks ? (p.n_chunks - (uint32_t)bid + nb - 1) / nb : 0u;
   it.vac0 = threadIdx.x < n_own ? __ldcg(&p.vacant[(uint32_t)bid + (uint32_t)nb * threadIdx.x]) : 0u;

@@ -146,6 +146,9 @@ struct Ctl {
   // next iteration takes, its secondary-buffer verdict, the last-block ticket
   // of the per-block vacancy scan, and the grid that scan was made for
   unsigned long long fill_take;
+  // every block takes quota_level of them, the first quota_extra one more
+  // (quota_level ~0: the per-block arrays hold the quotas)
+  unsigned int quota_level, quota_extra;
   unsigned int defer_local;
   unsigned int done_p;
   unsigned int local_blocks;
@@ -195,7 +198,6 @@ struct Params {
   int n_keys;
   uint32_t* perm;          // n_slots
   uint32_t* block_counts;  // live-key counts per counting block, (n_keys - 1) x blocks, key major
-  uint32_t* block_offsets; // their exclusive scan: each block's first position per key
   // geometry
   int n_layers;
   int n_materials;

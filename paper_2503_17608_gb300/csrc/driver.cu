@@ -541,7 +541,6 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
   // or the persistent grid
   const size_t max_blocks = p.n_tiles > 4096 ? p.n_tiles : 4096;
   CREATE_CUDA(dalloc(ctx, &p.block_counts, (size_t)kKeysFull * max_blocks));
-  CREATE_CUDA(dalloc(ctx, &p.block_offsets, (size_t)kKeysFull * max_blocks));
   CREATE_CUDA(dalloc(ctx, &p.block_vacant, (size_t)kMaxLoopBlocks));
   CREATE_CUDA(dalloc(ctx, &p.block_quota, (size_t)kMaxLoopBlocks));
   CREATE_CUDA(dalloc(ctx, &p.block_prefix, (size_t)kMaxLoopBlocks));

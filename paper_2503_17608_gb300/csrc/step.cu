@@ -682,11 +682,8 @@ __device__ void scan_vacancy(const Params& p) {
 }
 
 // Bookkeeping at the end of phase A, by one block: commit the initializers
-// taken, scan the per-(key, block) counts of the live keys (nb blocks counted
-// them) in key-major order into each block's first output position per key
-// and the key offsets, and decide whether this iteration's secondaries are
-// sure to fit.
-__device__ void bookkeeping_after_fill_step(const Params& p, bool did_fill, int nb) {
+// taken and decide whether this iteration's secondaries are sure to fit.
+__device__ void bookkeeping_after_fill_step(const Params& p, bool did_fill) {
   Ctl* c = p.ctl;
   if (did_fill && threadIdx.x == 0) {
     const unsigned long long queued = c->tail - c->head;
@@ -697,20 +694,6 @@ __device__ void bookkeeping_after_fill_step(const Params& p, bool did_fill, int 
     c->head += take;
     c->alive += take;
     c->total_vacant = tv - take;
-  }
-  if (global_partition(p.policy)) {
-    uint32_t* offs = p.block_offsets;
-    const int live_keys = p.n_keys - 1;  // the last key is the vacant one
-    const unsigned long long total = block_scan_counts(
-        p.block_counts, (uint32_t)(live_keys * nb), [offs](uint32_t i, unsigned long long v) { offs[i] = (uint32_t)v; });
-    __syncthreads();
-    if ((int)threadIdx.x < live_keys) c->offsets[threadIdx.x] = offs[threadIdx.x * nb];
-    if (threadIdx.x == 0) c->part_blocks = (unsigned)nb;
-    if ((int)threadIdx.x == live_keys) {
-      c->offsets[live_keys] = (unsigned)total;
-      c->offsets[p.n_keys] = p.n_slots;
-    }
-    __syncthreads();
   }
   if (threadIdx.x == 0) {
     const unsigned long long queued = c->tail - c->head;
@@ -782,12 +765,15 @@ __device__ void phase_fill_step(const Params& p, int bid, int nb, const SharedSt
   }
   if (bookkeeping && last_block_done(&c->done_a, nb)) {
     const long long t0 = clock64();
-    bookkeeping_after_fill_step(p, true, nb);
+    bookkeeping_after_fill_step(p, true);
     if (threadIdx.x == 0) c->book_total[0] += (unsigned long long)(clock64() - t0);
   }
 }
 
-// Scatter slot indices into the partition. Block b owns chunks b, b + nb,
+// Scatter slot indices into the partition. Every block sums the per-(key,
+// block) counts of the live keys itself, one warp per key, into its first
+// position per key (a scan by the last block of phase A held up all others,
+// 2.4 us per iteration); block 0 notes the key offsets. Block b owns chunks b, b + nb,
 // b + 2 nb, ... (the chunks it counted in phase A). It walks those that hold
 // live keys in that order, one per warp, and places each live slot at: the
 // block's first position for the key (from the scan) + the block's same-key
@@ -803,7 +789,34 @@ __device__ void phase_scatter(const Params& p, int bid, int nb) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = (int)(blockDim.x >> 5);
   const unsigned lt = (1u << lane) - 1u;
-  if ((int)threadIdx.x < live_keys) s_cursor[threadIdx.x] = p.block_offsets[threadIdx.x * nb + bid];
+  __shared__ unsigned s_tot[kMaxKeys], s_before[kMaxKeys];
+  for (int k = warp; k < live_keys; k += nwarps) {
+    unsigned tot = 0, bef = 0;
+    for (int i = lane; i < nb; i += 32) {
+      const unsigned v = __ldcg(&p.block_counts[k * nb + i]);
+      tot += v;
+      bef += i < bid ? v : 0u;
+    }
+    tot = __reduce_add_sync(0xffffffffu, tot);
+    bef = __reduce_add_sync(0xffffffffu, bef);
+    if (lane == 0) {
+      s_tot[k] = tot;
+      s_before[k] = bef;
+    }
+  }
+  __syncthreads();
+  if ((int)threadIdx.x <= live_keys) {
+    unsigned base = 0;
+    for (int k = 0; k < (int)threadIdx.x; ++k) base += s_tot[k];
+    if ((int)threadIdx.x < live_keys) s_cursor[threadIdx.x] = base + s_before[threadIdx.x];
+    if (bid == 0) {
+      p.ctl->offsets[threadIdx.x] = base;
+      if ((int)threadIdx.x == live_keys) {
+        p.ctl->offsets[p.n_keys] = p.n_slots;
+        p.ctl->part_blocks = (unsigned)nb;
+      }
+    }
+  }
   const uint32_t n_own = (uint32_t)bid < p.n_chunks ? (p.n_chunks - (uint32_t)bid + nb - 1) / nb : 0u;
   for (uint32_t m0 = 0; m0 < n_own; m0 += blockDim.x) {
     // this pass's live chunks of the block, compacted in order
@@ -1517,7 +1530,7 @@ __global__ void __launch_bounds__(kTile) k_pre_step(Params p) {
   const SharedStatic ss = carve_static(p, smem_raw);
   stage_static(p, ss);
   phase_fill_step(p, blockIdx.x, gridDim.x, ss, false, true, false);
-  if (last_block_done(&p.ctl->done_a, gridDim.x)) bookkeeping_after_fill_step(p, true, gridDim.x);
+  if (last_block_done(&p.ctl->done_a, gridDim.x)) bookkeeping_after_fill_step(p, true);
 }
 
 __global__ void k_along(Params p, int charged) {
@@ -1574,6 +1587,42 @@ __device__ __forceinline__ bool grid_barrier(const Params& p, unsigned nblocks,
   return s_ok != 0;
 }
 
+// End of a phase of the persistent loop: the last block to arrive runs `book`
+// (whole block) and lets the others go on; its ticket is the grid barrier,
+// so a phase costs one atomic per block instead of two. Waits are bounded as
+// grid_barrier's. With the partition's offsets summed by every block: 1 GeV
+// calorimeter sorted by action and type 4.37 -> 4.01 ms (36.3 -> 32.7 us per
+// iteration).
+template <class Book>
+__device__ __forceinline__ bool end_phase(const Params& p, unsigned* counter, unsigned nb, Book book) {
+  __shared__ unsigned s_last, s_gen;
+  __shared__ int s_ok;
+  unsigned int* gen = p.barrier + 1;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_gen = *reinterpret_cast<volatile unsigned*>(gen);
+    s_last = atomicAdd(counter, 1u) == nb - 1u ? 1u : 0u;
+    if (s_last) *reinterpret_cast<volatile unsigned*>(counter) = 0u;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    book();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_ok = *reinterpret_cast<volatile unsigned*>(p.barrier + 2) == 0u ? 1 : 0;
+      __threadfence();
+      atomicAdd(gen, 1u);
+    }
+  } else if (threadIdx.x == 0) {
+    s_ok = wait_generation(p, s_gen, kBarrierTimeoutCycles) ? 1 : 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
 // The whole step loop in one persistent cooperative launch: one block per
 // SM slot, the static tables staged into shared memory once, three grid
 // barriers per iteration (two without sorting).
@@ -1613,9 +1662,14 @@ __global__ void __launch_bounds__(kTile, 1) k_loop(Params p) {
       }
     }
     long long t0 = clock64();
-    phase_fill_step(p, bid, nb, ss, true, true, true);
+    phase_fill_step(p, bid, nb, ss, true, true, false);
     const long long wa = clock64() - t0;
-    if (!grid_barrier(p, nb)) break;
+    const bool ok_a = end_phase(p, &c->done_a, nb, [&] {
+      const long long tb = clock64();
+      bookkeeping_after_fill_step(p, true);
+      if (threadIdx.x == 0) c->book_total[0] += (unsigned long long)(clock64() - tb);
+    });
+    if (!ok_a) break;
     mark(0, wa);
     if (sorted) {
       t0 = clock64();
@@ -1625,9 +1679,15 @@ __global__ void __launch_bounds__(kTile, 1) k_loop(Params p) {
       mark(1, wb);
     }
     t0 = clock64();
-    phase_step(p, bid, nb, ss, true, 0, 0);
+    phase_step(p, bid, nb, ss, false, 0, 0);
     const long long wc = clock64() - t0;
-    if (!grid_barrier(p, nb)) break;
+    const bool ok_c = end_phase(p, &c->done_c, nb, [&] {
+      const long long tb = clock64();
+      scan_vacancy(p);
+      if (threadIdx.x < 32) loop_ctl_warp(p);
+      if (threadIdx.x == 0) c->book_total[1] += (unsigned long long)(clock64() - tb);
+    });
+    if (!ok_c) break;
     mark(2, wc);
     parity ^= 1u;
   }
