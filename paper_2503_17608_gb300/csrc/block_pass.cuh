@@ -237,7 +237,8 @@ __device__ __forceinline__ BlockIter load_block_iter(const Params& p, int bid, i
 // other blocks wait (bounded) for the last one to bump the generation word,
 // so an iteration costs one global atomic per block. Returns false if the
 // wait gave up (abort word set, ERR_BARRIER_TIMEOUT).
-__device__ bool end_block_pass(const Params& p, int bid, int nb, const BlockIter& it, long long vdelta, bool persistent,
+template <bool kPersistent>
+__device__ bool end_block_pass(const Params& p, int bid, int nb, const BlockIter& it, long long vdelta,
                                cudaGraphConditionalHandle handle, int use_handle, long long t_work0) {
   const unsigned long long head = it.head, take = it.take;
   __shared__ long long s_delta;
@@ -253,7 +254,7 @@ __device__ bool end_block_pass(const Params& p, int bid, int nb, const BlockIter
   __syncthreads();
   if (threadIdx.x == 0) {
     p.block_vacant[bid] = (uint32_t)((long long)it.vtot + s_delta);
-    if (persistent) {
+    if (kPersistent) {
       atomicMax(&c->iter_max[it.iteration & 1][2], (unsigned long long)(clock64() - t_work0));
       s_gen = *reinterpret_cast<volatile unsigned*>(gen);
     }
@@ -275,6 +276,7 @@ __device__ bool end_block_pass(const Params& p, int bid, int nb, const BlockIter
       c->head = head + take;
       c->alive += take;
     }
+    if (!kPersistent) copy_hits(p);
     load_block_vacancies(p, s_v, nb, &s_sum, &s_vmin, &s_vmax);
     if (threadIdx.x == 0) c->total_vacant = s_sum;
     __syncthreads();
@@ -283,17 +285,17 @@ __device__ bool end_block_pass(const Params& p, int bid, int nb, const BlockIter
     const unsigned long long planned = plan_block_quotas(p, s_v, nb, s_vmin, s_vmax, s_take, block_quota_cap(p.policy));
     if (threadIdx.x == 0) {
       if (planned != s_take) c->fill_take = planned;
-      if (use_handle) cudaGraphSetConditional(handle, c->cont);
+      if (!kPersistent && use_handle) cudaGraphSetConditional(handle, c->cont);
       c->book_total[1] += (unsigned long long)(clock64() - t0);
     }
     __syncthreads();
-    if (persistent && threadIdx.x == 0) {
+    if (kPersistent && threadIdx.x == 0) {
       __threadfence();
       atomicAdd(gen, 1u);
     }
     return true;
   }
-  if (!persistent) return true;
+  if (!kPersistent) return true;
   if (threadIdx.x == 0) {
     const bool ok = wait_generation(p, s_gen, kBarrierTimeoutCycles);
     __threadfence();
@@ -665,9 +667,9 @@ __device__ void local_pass(const Params& p, int bid, int nb, const SharedStatic&
 // fresh tracks over all SMs), then the end of the block's pass, where the
 // last block to finish commits the fill, scans the per-block and per-tile
 // vacancy counts and ends the iteration (which plans the next fill).
+template <bool kPersistent>
 __device__ bool block_iteration(const Params& p, int bid, int nb, const SharedStatic& ss,
-                                cudaGraphConditionalHandle handle, int use_handle, bool persistent,
-                                const BlockIter& it) {
+                                cudaGraphConditionalHandle handle, int use_handle, const BlockIter& it) {
   const long long t_work0 = clock64();
   Ctl* c = p.ctl;
   if (bid == 0 && threadIdx.x == 0 && !it.blocks_ok) atomicOr(&c->error, ERR_VACANCY);
@@ -681,7 +683,6 @@ __device__ bool block_iteration(const Params& p, int bid, int nb, const SharedSt
   flush_counter(&c->steps_iter, n.steps, false);
   flush_counter(&c->filled_total, n.fill, false);
   if (n.n_def) atomicAdd(&c->n_deferred, (unsigned)n.n_def);
-  return end_block_pass(p, bid, nb, it, (long long)n.killed - (long long)n.fill, persistent, handle, use_handle,
-                        t_work0);
+  return end_block_pass<kPersistent>(p, bid, nb, it, (long long)n.killed - (long long)n.fill, handle, use_handle, t_work0);
 }
 

@@ -23,6 +23,7 @@ constexpr double kNA = 6.02214076e23;
 constexpr double kNeWater = 3.343e23;  // reference electron density of the photon model
 constexpr double kZWater = 7.42;       // reference effective Z of the photon model
 constexpr int kTimingPool = 8192;
+constexpr uint64_t kMappedHits = 4096;   // tally values a kernel writes to pinned memory at the end of an iteration
 constexpr uint64_t kReadInPlace = 4096;  // staged primaries read by the device from pinned host memory
 
 uint64_t next_pow2(uint64_t v) {
@@ -75,6 +76,7 @@ struct celer_ctx {
   // per-iteration hit readout of the host loop: 0 off, 1 stream-ordered, 2 synchronous
   int hit_mode = 0;
   double* h_hits = nullptr;
+  double* hits_mapped = nullptr;  // h_hits as the device addresses it, if it is pinned and small
   double t_total_ms[KID_COUNT] = {};
   uint64_t t_launches[KID_COUNT] = {};
 };
@@ -545,10 +547,13 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
   CREATE_CUDA(dalloc(ctx, &p.block_quota, (size_t)kMaxLoopBlocks));
   CREATE_CUDA(dalloc(ctx, &p.block_prefix, (size_t)kMaxLoopBlocks));
   CREATE_CUDA(dalloc(ctx, &ctx->ring_state, (size_t)p.ring_capacity));
-  double* d_zb = nullptr;
-  int32_t* d_lmat = nullptr;
-  CREATE_CUDA(dalloc(ctx, &d_zb, L + 1));
-  CREATE_CUDA(dalloc(ctx, &d_lmat, L));
+  // the static tables, layer planes and layer materials in one run, as the
+  // kernels lay them out in shared memory (one bulk copy)
+  unsigned char* d_static = nullptr;
+  CREATE_CUDA(dalloc(ctx, &d_static, p.static_bytes));
+  double2* d_tables = reinterpret_cast<double2*>(d_static);
+  double* d_zb = reinterpret_cast<double*>(d_tables + (size_t)pb->n_materials * kCols * kGrid);
+  int32_t* d_lmat = reinterpret_cast<int32_t*>(d_zb + L + 1);
   CREATE_CUDA(cudaMemcpyAsync(d_zb, ctx->zb.data(), sizeof(double) * (L + 1), cudaMemcpyHostToDevice, ctx->stream));
   std::vector<int32_t> lm(ctx->layer_mat.begin(), ctx->layer_mat.end());
   CREATE_CUDA(cudaMemcpyAsync(d_lmat, lm.data(), sizeof(int32_t) * L, cudaMemcpyHostToDevice, ctx->stream));
@@ -566,10 +571,8 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
   CREATE_CUDA(dalloc(ctx, &p.trace, kTraceRows));
 
   // tables, built on the device
-  double2* d_tables = nullptr;
   double* d_scratch = nullptr;
   MaterialData* d_mats = nullptr;
-  CREATE_CUDA(dalloc(ctx, &d_tables, (size_t)pb->n_materials * kCols * kGrid));
   CREATE_CUDA(dalloc(ctx, &d_scratch, table_scratch_doubles(pb->n_materials)));
   CREATE_CUDA(dalloc(ctx, &d_mats, pb->n_materials));
   CREATE_CUDA(cudaMemcpyAsync(d_mats, mats.data(), sizeof(MaterialData) * mats.size(), cudaMemcpyHostToDevice,
@@ -790,10 +793,16 @@ celer_status celer_run_iterations(celer_ctx* ctx, int mode, uint64_t budget, uin
     int cur = 0;
     bool have_prev = false;
     const size_t hit_bytes = sizeof(double) * (size_t)ctx->p.max_events * (size_t)ctx->p.n_bins;
+    // (small pinned hit buffers are written by the iteration's last block)
+    ctx->p.hits = ctx->hit_mode == 1 ? ctx->hits_mapped : nullptr;
+    struct ClearHits {
+      Params& p;
+      ~ClearHits() { p.hits = nullptr; }
+    } clear_hits{ctx->p};
     for (;;) {
       for (int i = 0; i < batch; ++i) {
         launch_iteration(ctx, ctx->stream, 0, 0);
-        if (ctx->hit_mode == 1) {
+        if (ctx->hit_mode == 1 && !ctx->p.hits) {
           CELER_CUDA(ctx, cudaMemcpyAsync(ctx->h_hits, ctx->p.tally, hit_bytes, cudaMemcpyDeviceToHost, ctx->stream));
         } else if (ctx->hit_mode == 2) {
           // a synchronous copy: the whole device waits (every stream), then the
@@ -941,6 +950,14 @@ celer_status celer_set_hit_readout(celer_ctx* ctx, int mode, double* host_hits, 
     return fail(ctx, CELER_ERR_INVALID, "hit buffer missing or smaller than max_events x bins");
   ctx->hit_mode = mode;
   ctx->h_hits = mode ? host_hits : nullptr;
+  ctx->hits_mapped = nullptr;
+  if (mode == 1 && (uint64_t)ctx->p.max_events * (uint64_t)ctx->p.n_bins <= kMappedHits) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, host_hits) != cudaSuccess)
+      cudaGetLastError();  // not a CUDA pointer: copied
+    else if (at.type == cudaMemoryTypeHost && at.devicePointer)
+      ctx->hits_mapped = static_cast<double*>(at.devicePointer);
+  }
   return CELER_OK;
 }
 

@@ -417,12 +417,33 @@ __device__ __forceinline__ uint8_t step_limit(const Params& p, uint32_t slot, co
 //      interaction, in partition order; the last block to finish ends the
 //      iteration (counters, trace, loop condition).
 
+__device__ __forceinline__ bool static_arrived(unsigned bar) {
+  unsigned done;
+  asm volatile(
+      "{\n .reg .pred q;\n mbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(done)
+      : "r"(bar)
+      : "memory");
+  return done != 0u;
+}
+// (each try suspends the thread for a while; the limit is far above any copy)
+static __device__ __noinline__ void wait_static(const Params& p, unsigned bar) {
+  for (int i = 0; i < (1 << 20); ++i)
+    if (static_arrived(bar)) return;
+  atomicOr(&p.ctl->error, ERR_BARRIER_TIMEOUT);
+}
+
 // Static data every step kernel needs in shared memory: cross-section and
-// range tables, layer planes and layer materials.
+// range tables, layer planes and layer materials (one contiguous run of
+// static_bytes in device memory, laid out as here).
 struct SharedStatic {
   double2* tab;
   double* zb;
   int32_t* lmat;
+  unsigned bar;  // the copy's barrier (shared address)
+  __device__ __forceinline__ void ready(const Params& p) const {
+    if (!static_arrived(bar)) wait_static(p, bar);
+  }
 };
 
 __device__ __forceinline__ SharedStatic carve_static(const Params& p, unsigned char* raw) {
@@ -430,17 +451,36 @@ __device__ __forceinline__ SharedStatic carve_static(const Params& p, unsigned c
   s.tab = reinterpret_cast<double2*>(raw);
   s.zb = reinterpret_cast<double*>(s.tab + p.n_materials * kCols * kGrid);
   s.lmat = reinterpret_cast<int32_t*>(s.zb + p.n_layers + 1);
+  s.bar = 0u;
   return s;
 }
 
-__device__ __forceinline__ void stage_static(const Params& p, const SharedStatic& s) {
-  const int ntab = p.n_materials * kCols * kGrid;
-  for (int i = threadIdx.x; i < ntab; i += blockDim.x) s.tab[i] = p.tables[i];
-  for (int i = threadIdx.x; i <= p.n_layers; i += blockDim.x) s.zb[i] = p.zb[i];
-  for (int i = threadIdx.x; i < p.n_layers; i += blockDim.x) s.lmat[i] = p.layer_mat[i];
+// The copy of the static data into shared memory in the kernels launched every
+// iteration, one bulk copy (TMA): one thread starts it, ready() waits for it
+// (bounded) after the block's first loads (water cube in the graph loop 1.16 ->
+// 1.12 ms). Waiting only where the data are first used, in the bodies shared
+// with the persistent loops, cost those 3-4 %. Ends with a block barrier.
+__device__ __forceinline__ void stage_static(const Params& p, SharedStatic& s, unsigned long long* bar) {
+  s.bar = (unsigned)__cvta_generic_to_shared(bar);
+  if (threadIdx.x == 0) {
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(s.tab);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s.bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s.bar), "r"(p.static_bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(p.tables), "r"(p.static_bytes), "r"(s.bar)
+                 : "memory");
+  }
   __syncthreads();
 }
 
+// The same by every thread of the block, for the loops that do it once.
+__device__ __forceinline__ void stage_static(const Params& p, const SharedStatic& s) {
+  const uint4* src = reinterpret_cast<const uint4*>(p.tables);
+  uint4* dst = reinterpret_cast<uint4*>(s.tab);
+  for (uint32_t i = threadIdx.x; i < p.static_bytes / 16u; i += blockDim.x) dst[i] = src[i];
+  __syncthreads();
+}
 
 // Clear the per-iteration counters (one thread).
 __device__ __forceinline__ void clear_iteration_counters(Ctl* c) {
@@ -1357,6 +1397,17 @@ __device__ void loop_ctl_warp(const Params& p, unsigned long long* take_out = nu
   }
 }
 
+// The tally rows to pinned host memory at the end of an iteration (whole block,
+// after every other block's deposits): the hit copy of the host loop without
+// the gap of a copy between two kernels (event of 200 primaries, 128
+// iterations with a copy each: 4.94 -> 3.64 ms).
+static __device__ __noinline__ void copy_out_row(double* dst, const double* src, uint32_t n) {
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) dst[i] = __ldcg(src + i);
+}
+__device__ __forceinline__ void copy_hits(const Params& p) {
+  if (p.hits != nullptr) copy_out_row(p.hits, p.tally, p.max_events * (uint32_t)p.n_bins);
+}
+
 // Along-step and, if the step ends in one, the interaction of the track in
 // `slot` (phase C's body). Returns true if the track ended.
 __device__ __forceinline__ bool step_one(const Params& p, uint32_t slot, uint8_t st, const SharedStatic& ss, bool tight,
@@ -1427,6 +1478,7 @@ __device__ void phase_step(const Params& p, int bid, int nb, const SharedStatic&
   apply_fills(p, bid, nb);
   if (bookkeeping && last_block_done(&p.ctl->done_c, nb)) {
     const long long t0 = clock64();
+    copy_hits(p);
     scan_vacancy(p);
     if (threadIdx.x < 32) loop_ctl_warp(p);
     if (threadIdx.x == 0) {
@@ -1493,8 +1545,10 @@ __device__ void phase_post_only(const Params& p, uint8_t which, int bid, int nb)
 // Phase-merged launches (host loop / graph): A, B, C.
 __global__ void __launch_bounds__(kTile) k_fill_step(Params p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SharedStatic ss = carve_static(p, smem_raw);
-  stage_static(p, ss);
+  __shared__ unsigned long long s_bar;
+  SharedStatic ss = carve_static(p, smem_raw);
+  stage_static(p, ss, &s_bar);
+  ss.ready(p);
   phase_fill_step(p, blockIdx.x, gridDim.x, ss, true, true, true);
 }
 
@@ -1502,8 +1556,10 @@ __global__ void __launch_bounds__(kTile) k_scatter(Params p) { phase_scatter(p, 
 
 __global__ void k_step(Params p, cudaGraphConditionalHandle handle, int use_handle) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SharedStatic ss = carve_static(p, smem_raw);
-  stage_static(p, ss);
+  __shared__ unsigned long long s_bar;
+  SharedStatic ss = carve_static(p, smem_raw);
+  stage_static(p, ss, &s_bar);
+  ss.ready(p);
   phase_step(p, blockIdx.x, gridDim.x, ss, true, handle, use_handle);
 }
 
@@ -1511,10 +1567,12 @@ __global__ void k_step(Params p, cudaGraphConditionalHandle handle, int use_hand
 // as the loop).
 __global__ void __launch_bounds__(kTile) k_local(Params p, cudaGraphConditionalHandle handle, int use_handle) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SharedStatic ss = carve_static(p, smem_raw);
-  stage_static(p, ss);
+  __shared__ unsigned long long s_bar;
+  SharedStatic ss = carve_static(p, smem_raw);
+  stage_static(p, ss, &s_bar);
   const BlockIter it = load_block_iter(p, blockIdx.x, gridDim.x);
-  block_iteration(p, blockIdx.x, gridDim.x, ss, handle, use_handle, false, it);
+  ss.ready(p);
+  block_iteration<false>(p, blockIdx.x, gridDim.x, ss, handle, use_handle, it);
 }
 
 // Per-action launches: fill, step limit (+ bookkeeping), scatter, one
@@ -1527,16 +1585,20 @@ __global__ void __launch_bounds__(kTile) k_fill(Params p) {
 
 __global__ void __launch_bounds__(kTile) k_pre_step(Params p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SharedStatic ss = carve_static(p, smem_raw);
-  stage_static(p, ss);
+  __shared__ unsigned long long s_bar;
+  SharedStatic ss = carve_static(p, smem_raw);
+  stage_static(p, ss, &s_bar);
+  ss.ready(p);
   phase_fill_step(p, blockIdx.x, gridDim.x, ss, false, true, false);
   if (last_block_done(&p.ctl->done_a, gridDim.x)) bookkeeping_after_fill_step(p, true);
 }
 
 __global__ void k_along(Params p, int charged) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SharedStatic ss = carve_static(p, smem_raw);
-  stage_static(p, ss);
+  __shared__ unsigned long long s_bar;
+  SharedStatic ss = carve_static(p, smem_raw);
+  stage_static(p, ss, &s_bar);
+  ss.ready(p);
   phase_along_only(p, charged != 0, blockIdx.x, gridDim.x, ss);
 }
 
@@ -1544,6 +1606,7 @@ __global__ void k_post(Params p, int which) { phase_post_only(p, (uint8_t)which,
 
 __global__ void __launch_bounds__(kTile) k_loop_ctl(Params p, cudaGraphConditionalHandle handle, int use_handle) {
   apply_fills(p, 0, 1);
+  copy_hits(p);
   __syncthreads();
   scan_vacancy(p);
   if (threadIdx.x < 32) loop_ctl_warp(p);
@@ -1722,7 +1785,7 @@ __global__ void __launch_bounds__(kTile, 1) k_loop_local(Params p) {
       c->max_total[2] += c->iter_max[parity ^ 1u][2];
       c->iter_max[parity ^ 1u][2] = 0;
     }
-    const bool ok = block_iteration(p, bid, (int)nb, ss, 0, 0, true, it);
+    const bool ok = block_iteration<true>(p, bid, (int)nb, ss, 0, 0, it);
     if (!ok) break;
     if (bid == 0 && threadIdx.x == 0) {
       const long long now = clock64();
