@@ -24,7 +24,7 @@
 //    that they run the same code.
 // Against one crossing per piece with the tracks in the slot store: one event
 // of 12 particles 0.90 -> 0.68 ms, 1 GeV calorimeter 1.25 -> 1.05 ms, 4 T
-// calorimeter 10,000 x 10 GeV 3.50 -> 3.20 ms, 100,000 x 10 GeV 25.4 -> 18.5 ms.
+// calorimeter 10,000 x 10 GeV 3.50 -> 3.10 ms, 100,000 x 10 GeV 25.4 -> 15.9 ms.
 #pragma once
 
 // ---- the shared-memory track store of a block
@@ -780,16 +780,20 @@ __device__ __noinline__ void store_tracks(const Params& p, const TrackCache<kCap
 // Warps of a block that take pieces of any size; the others take full pieces
 // only: small pieces fetch the same instructions for fewer tracks. Measured
 // with 1, 2 and 3: 1 GeV calorimeter 1.41, 1.17 and 1.18 ms, 4 T calorimeter
-// 4.20, 3.49 and 3.53 ms.
+// 4.20, 3.49 and 3.53 ms. A block that holds kManyLive tracks always has a
+// full piece waiting (six kinds hold 186 in part-filled ones), and its job ends
+// later than its tracks' chains: there every warp takes full pieces only
+// (100,000 x 10 GeV 17.6 -> 15.9 ms; 16.4 from 512 tracks on, 15.9 from 850),
+// unless interactions wait for buffer space.
 constexpr int kAnyPieceWarps = 2;
 // Warps of a block that always look for work, and helpers beside them that
-// take full pieces only while the block holds at least kHelpLive tracks and a
+// take full pieces only while the block holds at least kManyLive tracks and a
 // kind kHelpWaiting of them: they hide each other's fetches where work abounds
 // (100,000 x 10 GeV 20.0 -> 18.6 ms), but slow down the chains of a smaller
 // job that runs beside them (10,000 x 10 GeV without the first condition 3.3
 // -> 4.0 ms).
 constexpr int kBaseWarps = 8, kWarpThreads = 512;
-constexpr unsigned kHelpWaiting = 64, kHelpLive = 640;
+constexpr unsigned kHelpWaiting = 64, kManyLive = 640;
 // A block with tracks waiting looks at the buffer this often at most (~2 us).
 constexpr unsigned kLookCycles = 4000;
 // Live tracks a block fills itself up to from the buffer while no full piece
@@ -957,9 +961,11 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     unsigned flags = 0;
     if (lane == 0)
       flags = (*reinterpret_cast<volatile unsigned*>(&s_exit) != 0u ? 1u : 0u) |
-              (*reinterpret_cast<volatile unsigned*>(&s_drain) != 0u ? 2u : 0u);
+              (*reinterpret_cast<volatile unsigned*>(&s_drain) != 0u ? 2u : 0u) |
+              (*reinterpret_cast<volatile unsigned*>(&s_live) >= kManyLive ? 4u : 0u) |
+              (*reinterpret_cast<volatile unsigned*>(&s_deferred) != 0u ? 8u : 0u);
     flags = __shfl_sync(0xffffffffu, flags, 0);
-    const bool drain = flags != 0u;
+    const bool drain = (flags & 3u) != 0u, many = (flags & 4u) != 0u, full_buffer = (flags & 8u) != 0u;
     if (helper && drain) break;
     // the kinds this round may take: all; draining, the pending interactions;
     // aborted, only those that need no buffer space
@@ -971,17 +977,18 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     long long t_read = 0, t_done = 0;
 #endif
     // Each of lanes 0..5 looks at one kind. Base warps below any_warps take
-    // pieces of any size, the others full ones only (while draining any warp
-    // takes any piece: a warp that leaves the loop may have been the last one
-    // allowed to take a small piece): with few tracks alive a block's work is
-    // concentrated in full warps instead of spread over many part-filled ones.
+    // pieces of any size unless the block holds many tracks, the others full
+    // ones only (while draining any warp takes any piece: a warp that leaves
+    // the loop may have been the last one allowed to take a small piece): with
+    // few tracks alive a block's work is concentrated in full warps instead of
+    // spread over many part-filled ones.
     unsigned waiting = 0;
     if (lane < kWarpKinds && ((allowed >> lane) & 1u)) {
       const unsigned hd = *reinterpret_cast<volatile unsigned*>(&s_head[lane]);  // before the tail: hd <= tail
       waiting = *reinterpret_cast<volatile unsigned*>(&s_tail[lane]) - hd;
     }
     constexpr unsigned kChargedKinds = (1u << W_ELECTRON) | (1u << W_MOLLER) | (1u << W_BREMS);
-    const bool any_size = drain || warp < any_warps;
+    const bool any_size = drain || (warp < any_warps && (!many || full_buffer));
     const unsigned full = __ballot_sync(0xffffffffu, waiting >= 32u), some = __ballot_sync(0xffffffffu, waiting > 0u);
     // The kind to take: of those waiting enough, for a warp of any-size pieces
     // charged tracks first (their steps carry a shower's longest chains of
@@ -997,8 +1004,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
                               : 0u;
     const unsigned picked = __reduce_max_sync(0xffffffffu, cand);
     const unsigned pick_k = picked != 0u ? 15u - (picked & 15u) : 0xFFu;
-    if (helper && (picked == 0u || ((picked >> 4) & 0xFFFFFu) < kHelpWaiting ||
-                   *reinterpret_cast<volatile unsigned*>(&s_live) < kHelpLive)) {
+    if (helper && (picked == 0u || ((picked >> 4) & 0xFFFFFu) < kHelpWaiting || !many)) {
       if (events != 0u) flush_warp_counts(p, steps, killed, fill);
       events = 0u;
       __nanosleep(10000);
@@ -1017,7 +1023,6 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     uint32_t load_chunk = 0xFFFFFFFFu;  // a chunk of parked tracks to load
     // (interactions wait for buffer space: entries must be taken whatever the
     // target, or no block would make room for another)
-    const bool full_buffer = *reinterpret_cast<volatile unsigned*>(&s_deferred) != 0u;
     bool look = !drain && !helper && (scarce || full_buffer);
     if (look && some != 0u)  // work waits here: look at the buffer every kLookCycles at most
       look = (unsigned)clock64() - *reinterpret_cast<volatile unsigned*>(&s_looked) > kLookCycles;

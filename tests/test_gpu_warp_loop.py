@@ -107,3 +107,14 @@ def test_queued_primaries_between_runs_of_all_loops(n):
         o = run_oracle(prob, prim)
         np.testing.assert_array_equal(hist["steps"][k * n:(k + 1) * n], o["hist"]["steps"])
         np.testing.assert_allclose(edep[k * n:(k + 1) * n], o["edep"], rtol=1e-9, atol=1e-9 * 10.0)
+
+
+@pytest.mark.parametrize("n,energy", [(96000, 5.0), (120000, 20.0), (160000, 1.0)])
+def test_blocks_that_hold_many_tracks(n, energy):
+    """640 tracks a block and more (97,280 on 152 blocks): only full pieces are
+    taken until the number falls below it, small ones after that."""
+    prob = wl.calorimeter_problem(1 << 18, Bz=4.0, init_capacity=1 << 18, history_capacity=n, sort_policy=wl.SORT_LOCAL)
+    prim = wl.electron_beam(n, energy, patch_half=5.0)
+    prim["ptype"][1::2] = wl.GAMMA
+    g = run_gpu(prob, prim, mode=binding.LOOP_ASYNC)
+    oracle_check(prob, prim, g["hist"], g["edep"])
