@@ -44,6 +44,7 @@ __global__ void k_async_prepare(Params p) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     p.ctl->finished = head - p.ctl->alive;
     p.ctl->avail = tail - head;
+    p.ctl->room = (long long)(p.ring_capacity - (tail - head));
     p.ctl->async_passes = 0;
     p.ctl->vacant_seen = 0;
     p.ctl->done_x = 0u;
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(kTile, 1) k_loop_async(Params p) {
           if (old >= (long long)want) {
             take = (unsigned)want;
             first = atomicAdd(&c->head, want);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&c->room), want);
           } else {
             atomicAdd(&c->avail, want);
           }

@@ -157,6 +157,7 @@ struct Ctl {
   // tail), the most block passes any block ran, and the exit ticket
   unsigned long long finished;
   unsigned long long avail;          // written entries not yet claimed by a reader (may dip below 0 briefly)
+  long long room;                    // entries free for a writer (may dip below 0 briefly)
   unsigned long long async_passes;
   unsigned long long vacant_seen;    // vacant slots the blocks of a per-warp run counted at its start
   unsigned int done_x;

@@ -8,7 +8,7 @@ import pytest
 
 from paper_2503_17608_gb300 import binding, workloads as wl
 
-from gpu_helpers import match_fraction, run_gpu, run_oracle
+from gpu_helpers import assert_conservation, match_fraction, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -118,3 +118,15 @@ def test_blocks_that_hold_many_tracks(n, energy):
     prim["ptype"][1::2] = wl.GAMMA
     g = run_gpu(prob, prim, mode=binding.LOOP_ASYNC)
     oracle_check(prob, prim, g["hist"], g["edep"])
+
+
+@pytest.mark.parametrize("policy", [wl.SORT_LOCAL, wl.SORT_DATA])
+@pytest.mark.parametrize("capacity", [4096, 8192, 16384])
+def test_buffer_smaller_than_the_shower(policy, capacity):
+    """The buffer's free entries run out: groups of lanes get none or some of
+    what they ask for, and the interactions without one wait for room."""
+    prob = wl.calorimeter_problem(1 << 15, Bz=4.0, init_capacity=capacity, sort_policy=policy)
+    prim = wl.electron_beam(3000, 200.0, patch_half=5.0)
+    g = run_gpu(prob, prim, mode=binding.LOOP_ASYNC)
+    oracle_check(prob, prim, g["hist"], g["edep"])
+    assert_conservation(prim, g["tally"], rel=1e-11)
