@@ -125,7 +125,8 @@ struct Ctl {
   unsigned int defer;                // 1: secondary-producing kernels postpone this iteration
   unsigned int n_deferred;
   unsigned int error;
-  unsigned int cont;                 // 1 while alive + queued > 0
+  unsigned int cont;                 // the run goes on: tracks left, no error, iterations left in its budget
+  unsigned int pending;              // alive + queued > 0 at the end of the last iteration (1 as a run begins)
   unsigned int stall;                // consecutive iterations without progress
   unsigned int done_a, done_c;       // last-block tickets of the fill/step-limit and step phases
   unsigned long long total_vacant;   // vacant slots (scanned at the end of an iteration)

@@ -34,13 +34,19 @@ struct LaunchShape {
 
 cudaError_t configure_kernels(const Params& p, int block, LaunchShape* shape);
 
+// How an iteration is launched: its last kernel sets the loop's graph handle;
+// its kernels do nothing once the run is over (in the graph, where several
+// iterations are unrolled), or once no track is left (in the host loop, whose
+// launches run ahead of the condition it reads back).
+enum IterMode : int { ITER_ALWAYS = 0, ITER_SET_HANDLE = 1, ITER_IF_CONT = 2, ITER_IF_PENDING = 4 };
+
 // phase-merged launches
-void launch_fill_step(const Params& p, const LaunchShape& sh, cudaStream_t s);
-void launch_scatter(const Params& p, const LaunchShape& sh, cudaStream_t s);
-void launch_step(const Params& p, const LaunchShape& sh, unsigned long long handle, int use_handle, cudaStream_t s);
+void launch_fill_step(const Params& p, const LaunchShape& sh, int mode, cudaStream_t s);
+void launch_scatter(const Params& p, const LaunchShape& sh, int mode, cudaStream_t s);
+void launch_step(const Params& p, const LaunchShape& sh, unsigned long long handle, int mode, cudaStream_t s);
 // block-local policy: one launch per iteration, and the per-block vacancy
 // scan a run starts with (both on the loop's grid)
-void launch_local(const Params& p, const LaunchShape& sh, unsigned long long handle, int use_handle, cudaStream_t s);
+void launch_local(const Params& p, const LaunchShape& sh, unsigned long long handle, int mode, cudaStream_t s);
 void launch_local_prepare(const Params& p, const LaunchShape& sh, cudaStream_t s);
 // per-tile vacancy scan for a slot-order run after block-local iterations
 void launch_scan_tiles(const Params& p, cudaStream_t s);
