@@ -126,7 +126,6 @@ struct Ctl {
   unsigned int n_deferred;
   unsigned int error;
   unsigned int cont;                 // the run goes on: tracks left, no error, iterations left in its budget
-  unsigned int pending;              // alive + queued > 0 at the end of the last iteration (1 as a run begins)
   unsigned int stall;                // consecutive iterations without progress
   unsigned int done_a, done_c;       // last-block tickets of the fill/step-limit and step phases
   unsigned long long total_vacant;   // vacant slots (scanned at the end of an iteration)
@@ -158,7 +157,6 @@ struct Ctl {
   // tail), the most block passes any block ran, and the exit ticket
   unsigned long long finished;
   unsigned long long avail;          // written entries not yet claimed by a reader (may dip below 0 briefly)
-  long long room;                    // entries free for a writer (may dip below 0 briefly)
   unsigned long long async_passes;
   unsigned long long vacant_seen;    // vacant slots the blocks of a per-warp run counted at its start
   unsigned int done_x;
@@ -166,6 +164,8 @@ struct Ctl {
   // last-block ticket of the push
   unsigned int push_bad;
   unsigned int done_push;
+  unsigned int pending;              // alive + queued > 0 at the end of the last iteration (1 as a run begins)
+  long long room;                    // asynchronous loop: entries free for a writer (may dip below 0 briefly)
 };
 
 struct TraceRow {
