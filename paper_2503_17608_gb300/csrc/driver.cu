@@ -544,9 +544,14 @@ celer_status celer_create(const celer_problem* pb, celer_ctx** out) {
       pre[t] = run;
       run += tvac[t];
     }
-    CREATE_CUDA(cudaMemcpy(p.vacant, vac.data(), sizeof(uint32_t) * p.n_chunks, cudaMemcpyHostToDevice));
-    CREATE_CUDA(cudaMemcpy(p.tile_vacant, tvac.data(), sizeof(uint32_t) * p.n_tiles, cudaMemcpyHostToDevice));
-    CREATE_CUDA(cudaMemcpy(p.tile_prefix, pre.data(), sizeof(unsigned long long) * p.n_tiles, cudaMemcpyHostToDevice));
+    // (on the context's stream, after the arrays' clearing there: a stream that
+    // does not wait for the default one may still be at an earlier array)
+    CREATE_CUDA(cudaMemcpyAsync(p.vacant, vac.data(), sizeof(uint32_t) * p.n_chunks, cudaMemcpyHostToDevice, ctx->stream));
+    CREATE_CUDA(cudaMemcpyAsync(p.tile_vacant, tvac.data(), sizeof(uint32_t) * p.n_tiles, cudaMemcpyHostToDevice,
+                                ctx->stream));
+    CREATE_CUDA(cudaMemcpyAsync(p.tile_prefix, pre.data(), sizeof(unsigned long long) * p.n_tiles, cudaMemcpyHostToDevice,
+                                ctx->stream));
+    CREATE_CUDA(cudaStreamSynchronize(ctx->stream));  // the vectors end here
   }
   CREATE_CUDA(dalloc(ctx, &p.perm, N));
   // per-(key, block) partition counts: blocks of phase A, at most one per tile

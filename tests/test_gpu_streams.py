@@ -98,3 +98,24 @@ def test_hit_readout_and_grid_arguments():
             ctx.run_events(mode)
             tally, esc = ctx.read_tallies(0)
             assert tally.sum() + esc == pytest.approx(evs[0]["E"].sum(), rel=1e-12)
+
+
+@pytest.mark.parametrize("policy,mode", [(wl.SORT_LOCAL, binding.LOOP_HOST), (wl.SORT_NONE, binding.LOOP_PERSISTENT)])
+def test_large_context_on_its_own_stream(policy, mode):
+    """Every slot of a new context is vacant, however long the clearing of its
+    arrays takes on a stream that does not wait for the default one."""
+    import torch
+
+    prim = wl.water_cube_primaries(200)
+    small = wl.water_cube_problem(n_slots=4096, sort_policy=policy)
+    with binding.Context(small) as ctx:
+        ctx.add_primaries(0, prim)
+        ctx.run_events(binding.LOOP_PERSISTENT)
+        want = ctx.stats()["steps_total"]
+    prob = small.replace(n_slots=1 << 21, init_capacity=1 << 24)
+    for _ in range(3):
+        stream = torch.cuda.Stream()
+        with binding.Context(prob, stream=stream.cuda_stream) as ctx:
+            ctx.add_primaries(0, prim)
+            ctx.run_events(mode)
+            assert ctx.stats()["steps_total"] == want
