@@ -429,12 +429,16 @@ def run_ours(args):
                  dict(value=r["steps"] / (r["ms"] / 1e3), ms_per_step=r["ms"] / args.steps,
                       track_steps_per_job=r["steps"] / args.steps / world)
                  for (p, m), r in results.items()}
-    # per job: primaries push, run start, (block-pass policies: per-block
-    # vacancy scan; asynchronous loop: buffer entry states), loop kernel
-    if loop.startswith("async"):
+    # per job: event reset, check and push of the primaries, the loop kernel,
+    # the control block's copy out; unless the run before left the state the
+    # per-warp loop starts from, the run start, too (block-pass policies:
+    # per-block vacancy scan; asynchronous loop: buffer entry states)
+    if loop == "async-warps":
         launches_per_job = 5
+    elif loop == "async":
+        launches_per_job = 8
     elif loop == "persistent":
-        launches_per_job = 4 if headline in block_pass else 3
+        launches_per_job = 7 if headline in block_pass else 6
     else:
         launches_per_job = None
     line = {
@@ -805,29 +809,31 @@ def load_peaks():
 # summaries under profiles/, one per kernel and workload). DRAM bytes per
 # launch come from one-pass full-size captures of the per-warp kernel on the
 # two calorimeters; other kernels report no traffic. Keys: (workload, policy), and
-# (workload, policy, loop) for the asynchronous loop kernel.
+# (workload, policy, loop) for the asynchronous loop's kernels (k_loop_async,
+# and k_loop_warps for per-warp scheduling; the roofline names both by the
+# first).
 BYTES_PER_STEP = 160.0
-FP64_FLOP_PER_STEP = {("calorimeter-1gev", "none"): 97.0, ("calorimeter-1gev", "action"): 97.0,
-                      ("calorimeter-1gev", "action_type"): 97.0, ("calorimeter-1gev", "data"): 86.4,
-                      ("calorimeter-1gev", "local"): 86.4, ("calorimeter-1gev", "local", "async-warps"): 86.5,
-                      ("calorimeter-field-10gev", "none"): 95.7, ("calorimeter-field-10gev", "action"): 95.7,
-                      ("calorimeter-field-10gev", "action_type"): 95.7, ("calorimeter-field-10gev", "data"): 92.5,
-                      ("calorimeter-field-10gev", "local"): 92.5,
+FP64_FLOP_PER_STEP = {("calorimeter-1gev", "none"): 81.4, ("calorimeter-1gev", "action"): 81.4,
+                      ("calorimeter-1gev", "action_type"): 81.4, ("calorimeter-1gev", "data"): 70.9,
+                      ("calorimeter-1gev", "local"): 70.9, ("calorimeter-1gev", "local", "async-warps"): 67.8,
+                      ("calorimeter-field-10gev", "none"): 79.6, ("calorimeter-field-10gev", "action"): 79.6,
+                      ("calorimeter-field-10gev", "action_type"): 79.6, ("calorimeter-field-10gev", "data"): 76.3,
+                      ("calorimeter-field-10gev", "local"): 76.3,
                       # the 4 T workload's counts come from its smaller case (2,500
                       # primaries, 2^18 slots; the op counters take 3 passes)
-                      ("calorimeter-field-10gev", "local", "async-warps"): 92.5,
+                      ("calorimeter-field-10gev", "local", "async-warps"): 70.8,
                       # water cube: k_loop (none; action and action_type run the same
-                      # kernel and counted the same on the calorimeters) and the others
-                      ("water-cube-10mev", "none"): 290.5, ("water-cube-10mev", "action"): 290.5,
-                      ("water-cube-10mev", "action_type"): 290.5, ("water-cube-10mev", None): 286.7}
-DRAM_BYTES_PER_LAUNCH = {("calorimeter-field-10gev", "local", "async-warps"): 49.74e6,
-                         ("calorimeter-1gev", "local", "async-warps"): 3.39e6}
+                      # kernel, and the block-pass kernels the same physics) and the
+                      # per-warp loop
+                      ("water-cube-10mev", None): 232.4, ("water-cube-10mev", "local", "async-warps"): 321.1}
+DRAM_BYTES_PER_LAUNCH = {("calorimeter-field-10gev", "local", "async-warps"): 22.88e6,
+                         ("calorimeter-1gev", "local", "async-warps"): 0.92e6}
 # FP64 warp instructions per track-step (sm__inst_executed_pipe_fp64 / track-steps)
 # of the loop kernel's one-launch ncu captures: an FP64 warp instruction holds
 # its sub-partition's FP64 pipe for 64 cycles whatever its active lanes, so
 # these set how busy the FP64 pipe is at a measured track-step rate.
-FP64_WARP_INSTR_PER_STEP = {("calorimeter-field-10gev", "local", "async-warps"): 3.36,
-                            ("calorimeter-1gev", "local", "async-warps"): 8.04}
+FP64_WARP_INSTR_PER_STEP = {("calorimeter-field-10gev", "local", "async-warps"): 3.09,
+                            ("calorimeter-1gev", "local", "async-warps"): 7.54}
 FP64_PIPE_CYCLES_PER_WARP_INSTR = 64.0
 # FP64 peak of GB300 derived from its unit counts: 2 DFMA per SM-cycle
 # (ncu peak_sustained) x 152 SMs x 2.07 GHz x 2 flop

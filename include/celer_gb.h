@@ -222,8 +222,9 @@ celer_status celer_step(celer_ctx* ctx, celer_step_stats* stats);
 /* Loop modes of celer_run_events. */
 enum {
   CELER_LOOP_HOST = 0,       /* host loop of per-iteration launches, polling the counters every few iterations */
-  CELER_LOOP_GRAPH = 1,      /* the iteration captured once into a CUDA graph whose conditional while-node
-                                repeats it on the device with no host round trip */
+  CELER_LOOP_GRAPH = 1,      /* iterations captured once into a CUDA graph whose conditional while-node
+                                repeats them on the device with no host round trip (four per round; those
+                                past the run's end do nothing) */
   CELER_LOOP_PERSISTENT = 2, /* one cooperative launch that runs every iteration: one block per SM slot,
                                 tables staged into shared memory once, phases separated by grid barriers
                                 whose waits are bounded (about 1 s, then CELER_ERR_TIMEOUT) */
@@ -238,8 +239,8 @@ enum {
                                 grows by the most passes any block ran (pieces any warp ran, with per-warp
                                 scheduling, celer_set_async_warps). With a budget (celer_run_iterations) a
                                 block stops after that many passes, or, per warp, the block drains once a
-                                warp has run that many pieces: its queued tracks take their step without a
-                                new step limit, so every track ends the run between two steps, as after a
+                                warp has run that many pieces: pending interactions are run and no further
+                                step is begun, so every track ends the run between two steps, as after a
                                 synchronous iteration. Waits are bounded: if no track steps for about 1 s
                                 the run ends with CELER_ERR_TIMEOUT or CELER_ERR_CAPACITY. */
 };
@@ -349,8 +350,9 @@ celer_status celer_set_parent_reuse(celer_ctx* ctx, int on);
  * soon as its own step is done instead of waiting for its block's slowest
  * group. Charged tracks are taken before photons (their steps form a shower's
  * longest chains), and in runs without an iteration budget all but the first
- * two warps of a block take only full pieces of 32 (budgeted runs, such as a
- * serving loop's chunks, let every warp take any piece). A block keeps its
+ * two warps of a block take only full pieces of 32, and all of them while the
+ * block holds many tracks (budgeted runs, such as a serving loop's chunks, let
+ * every warp take any piece otherwise). A block keeps its
  * live tracks in shared memory, at most 1024 of them (256 with more than four
  * materials); a block that starts a run with more steps them in turns.
  * Histories do not change. On by default. Takes effect at the next run. on outside
