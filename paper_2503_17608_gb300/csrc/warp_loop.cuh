@@ -967,7 +967,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     flags = __shfl_sync(0xffffffffu, flags, 0);
     const bool drain = (flags & 3u) != 0u, many = (flags & 4u) != 0u, full_buffer = (flags & 8u) != 0u;
     if (helper && drain) break;
-    // the kinds this round may take: all; draining, the pending interactions;
+    // the kinds to choose from now: all; draining, the pending interactions;
     // aborted, only those that need no buffer space
     const unsigned allowed = (flags & 1u) ? (1u << W_COMPTON)
                                           : (drain ? (1u << W_COMPTON) | (1u << W_PAIR) | (1u << W_MOLLER) | (1u << W_BREMS)
