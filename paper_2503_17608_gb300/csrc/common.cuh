@@ -234,7 +234,8 @@ struct Params {
   double* hist_escaped;
   double* hist_edep;       // hist_cap * n_bins
   TraceRow* trace;
-  double* hits;              // host loop with stream-ordered hit copies: the tally rows go here (pinned host
+  unsigned* cont_out;      // host loop: the loop condition after every iteration (pinned host memory), or null
+  double* hits;            // host loop with stream-ordered hit copies: the tally rows go here (pinned host
                              // memory) at the end of every iteration; null otherwise
 };
 

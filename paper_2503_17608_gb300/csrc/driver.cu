@@ -801,20 +801,28 @@ celer_status celer_run_iterations(celer_ctx* ctx, int mode, uint64_t budget, uin
     CELER_CUDA(ctx, cudaGetLastError());
     CELER_CUDA(ctx, launch_loop_async(pa, ctx->shape, ctx->stream));
   } else {
-    // Host loop: launch batches of iterations; before each new batch, look at
-    // the loop condition copied back after the batch before the previous one,
-    // so that the GPU never waits for the host.
+    // Host loop (a copy of the condition per batch, with the gap it left between
+    // two kernels: event of 200 primaries 3.01 ms, written by the kernels 2.86
+    // ms): launch batches of iterations; before each new batch, look at
+    // the loop condition that the kernels have written to pinned memory by the
+    // end of the batch before the previous one, so that the GPU never waits for
+    // the host.
     const int batch = 8;
     int cur = 0;
     bool have_prev = false;
     const size_t hit_bytes = sizeof(double) * (size_t)ctx->p.max_events * (size_t)ctx->p.n_bins;
     // (small pinned hit buffers are written by the iteration's last block)
     ctx->p.hits = ctx->hit_mode == 1 ? ctx->hits_mapped : nullptr;
-    struct ClearHits {
+    struct ClearOutputs {
       Params& p;
-      ~ClearHits() { p.hits = nullptr; }
-    } clear_hits{ctx->p};
+      ~ClearOutputs() {
+        p.hits = nullptr;
+        p.cont_out = nullptr;
+      }
+    } clear_outputs{ctx->p};
     for (;;) {
+      ctx->h_cont[cur] = 1u;  // (the batch that last wrote here has been waited for)
+      ctx->p.cont_out = ctx->h_cont + cur;
       for (int i = 0; i < batch; ++i) {
         launch_iteration(ctx, ctx->stream, 0, ITER_IF_PENDING);
         if (ctx->hit_mode == 1 && !ctx->p.hits) {
@@ -827,13 +835,11 @@ celer_status celer_run_iterations(celer_ctx* ctx, int mode, uint64_t budget, uin
         }
       }
       CELER_CUDA(ctx, cudaGetLastError());
-      CELER_CUDA(ctx, cudaMemcpyAsync(&ctx->h_cont[cur], &ctx->p.ctl->cont, sizeof(unsigned), cudaMemcpyDeviceToHost,
-                                      ctx->stream));
       CELER_CUDA(ctx, cudaEventRecord(ctx->cont_ev[cur], ctx->stream));
       if (have_prev) {
         const int prev = cur ^ 1;
         CELER_CUDA(ctx, cudaEventSynchronize(ctx->cont_ev[prev]));
-        if (ctx->h_cont[prev] == 0u) break;
+        if (*reinterpret_cast<volatile unsigned*>(ctx->h_cont + prev) == 0u) break;
       }
       have_prev = true;
       cur ^= 1;

@@ -1402,8 +1402,10 @@ __device__ void loop_ctl_warp(const Params& p, unsigned long long* take_out = nu
     }
     if (pending && it >= max_iterations) err |= ERR_ITERATIONS;
     if (err != error) c->error = err;
-    c->cont = (pending && err == 0u && it < budget_end) ? 1u : 0u;
+    const unsigned cont = (pending && err == 0u && it < budget_end) ? 1u : 0u;
+    c->cont = cont;
     c->pending = pending ? 1u : 0u;
+    if (p.cont_out) *reinterpret_cast<volatile unsigned*>(p.cont_out) = cont;
     c->steps_iter = 0;
     c->n_deferred = 0;
     const unsigned long long take = plan_local_fill(p, head, tail, alive, total_vacant);
