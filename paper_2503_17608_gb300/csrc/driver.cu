@@ -72,6 +72,7 @@ struct celer_ctx {
   // the entry states and counters of the asynchronous loop are as its next run
   // needs them, and h_ctl's iteration count is the device's (k_async_prepare)
   bool async_ready = false;
+  uint32_t live_rows = 0;  // event_live counts that read_ctl brings along, to h_bounce
   bool tiles_stale = false;  // the per-tile vacancy prefix predates the last block-local iterations
   // per-iteration hit readout of the host loop: 0 off, 1 stream-ordered, 2 synchronous
   int hit_mode = 0;
@@ -309,7 +310,8 @@ cudaError_t copy_out(celer_ctx* ctx, void* dst, const void* src, size_t bytes, v
 
 celer_status read_ctl(celer_ctx* ctx) {
   static_assert(sizeof(Ctl) % 4 == 0, "copied by words");
-  CELER_CUDA(ctx, copy_out(ctx, ctx->h_ctl, ctx->p.ctl, sizeof(Ctl)));
+  CELER_CUDA(ctx, copy_out(ctx, ctx->h_ctl, ctx->p.ctl, sizeof(Ctl), ctx->h_bounce, ctx->p.event_live,
+                           sizeof(uint32_t) * ctx->live_rows));
   CELER_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   ctx->stage_used = 0;
   ctx->ctl_fresh = true;
@@ -1222,3 +1224,37 @@ celer_status celer_debug_table(celer_ctx* ctx, int mat, int col, double* out) {
 }
 
 }  // extern "C"
+
+// Used by serve.cu: a run whose last read-back brings the live counts of the
+// events' rows along, and the tallies and escaped energy of several events
+// (n_bins + 1 values each) with one wait for all.
+__attribute__((visibility("hidden"))) celer_status run_and_read_live(celer_ctx* ctx, int mode, uint64_t budget,
+                                                                     uint64_t* done, uint32_t rows, uint32_t* live) {
+  const size_t bytes = sizeof(uint32_t) * (size_t)rows;
+  const bool along = bytes <= ctx->bounce_bytes;
+  ctx->live_rows = along ? rows : 0u;
+  const celer_status st = celer_run_iterations(ctx, mode, budget, done);
+  ctx->live_rows = 0u;
+  if (st != CELER_OK) return st;
+  if (!along) return celer_read_event_live(ctx, 0, rows, live);
+  std::memcpy(live, ctx->h_bounce, bytes);
+  return CELER_OK;
+}
+
+__attribute__((visibility("hidden"))) celer_status read_tallies_of(celer_ctx* ctx, const uint32_t* events, size_t n,
+                                                                   double* out) {
+  const size_t nb = (size_t)ctx->p.n_bins, width = nb + 1, per_wait = ctx->bounce_bytes / (sizeof(double) * width);
+  for (size_t k = 0; k < n;) {
+    const size_t m = n - k < per_wait ? n - k : per_wait;
+    for (size_t j = 0; j < m; ++j) {
+      const uint32_t row = events[k + j] % ctx->p.max_events;
+      double* const to = ctx->h_bounce + j * width;
+      CELER_CUDA(ctx, copy_out(ctx, to, ctx->p.tally + (size_t)row * nb, sizeof(double) * nb, to + nb,
+                               ctx->p.escaped + row, sizeof(double)));
+    }
+    CELER_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    std::memcpy(out + k * width, ctx->h_bounce, sizeof(double) * width * m);
+    k += m;
+  }
+  return CELER_OK;
+}

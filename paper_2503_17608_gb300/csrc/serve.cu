@@ -31,6 +31,10 @@ struct InFlight {
 
 }  // namespace
 
+// driver.cu
+celer_status run_and_read_live(celer_ctx* ctx, int mode, uint64_t budget, uint64_t* done, uint32_t rows, uint32_t* live);
+celer_status read_tallies_of(celer_ctx* ctx, const uint32_t* events, size_t n, double* out);
+
 extern "C" celer_status celer_serve(celer_ctx* ctx, const celer_request* reqs, uint64_t n,
                                     const celer_serve_options* opt_in, celer_request_result* results,
                                     celer_serve_summary* summary) {
@@ -62,8 +66,9 @@ extern "C" celer_status celer_serve(celer_ctx* ctx, const celer_request* reqs, u
   const double capacity = (double)(n_slots + ring);
   std::vector<uint8_t> row_busy(max_events, 0);
   std::vector<uint32_t> live(max_events, 0);
-  std::vector<double> tally(n_bins);
-  std::vector<InFlight> inflight;
+  std::vector<double> tallies;
+  std::vector<uint32_t> ended;
+  std::vector<InFlight> inflight, staying;
   double reserved = 0.0;
 
   for (uint64_t i = 0; i < n; ++i) {
@@ -107,37 +112,41 @@ extern "C" celer_status celer_serve(celer_ctx* ctx, const celer_request* reqs, u
       if (wait > 2e-4) std::this_thread::sleep_for(std::chrono::duration<double>(wait - 1e-4));
       continue;
     }
-    // a chunk of step iterations over every resident track
+    // A chunk of step iterations over every resident track, with the rows' live
+    // counts; then the tallies of all events that ended in it with one wait (a
+    // wait for the counts and one per event before: a burst of 32 events of 200
+    // particles 4.00 -> 3.71 ms).
     uint64_t done = 0;
-    s = celer_run_iterations(ctx, opt.mode, opt.chunk_iterations, &done);
+    s = run_and_read_live(ctx, opt.mode, opt.chunk_iterations, &done, (uint32_t)max_events, live.data());
     if (s != CELER_OK) return s;
     ++chunks;
-    // collect finished events
-    s = celer_read_event_live(ctx, 0, (uint32_t)max_events, live.data());
+    ended.clear();
+    for (const InFlight& f : inflight)
+      if (live[f.row] == 0u) ended.push_back(reqs[f.req].event);
+    tallies.resize(ended.size() * (n_bins + 1));
+    s = read_tallies_of(ctx, ended.data(), ended.size(), tallies.data());
     if (s != CELER_OK) return s;
-    for (size_t k = 0; k < inflight.size();) {
-      const InFlight f = inflight[k];
+    const double* tally = tallies.data();
+    staying.clear();
+    for (const InFlight& f : inflight) {
       if (live[f.row] != 0u) {
-        ++k;
+        staying.push_back(f);
         continue;
       }
-      double esc = 0.0;
-      s = celer_read_tallies(ctx, reqs[f.req].event, tally.data(), n_bins, &esc);
-      if (s != CELER_OK) return s;
       double sum = 0.0;
-      for (double v : tally) sum += v;
+      for (uint64_t b = 0; b < n_bins; ++b) sum += tally[b];
       celer_request_result& r = results[f.req];
       r.done_s = seconds_since(t0);
       r.edep = sum;
-      r.escaped = esc;
-      if (opt.tallies_out) std::memcpy(opt.tallies_out + f.req * n_bins, tally.data(), sizeof(double) * n_bins);
+      r.escaped = tally[n_bins];
+      if (opt.tallies_out) std::memcpy(opt.tallies_out + f.req * n_bins, tally, sizeof(double) * n_bins);
+      tally += n_bins + 1;
       last_done = r.done_s;
       row_busy[f.row] = 0;
       reserved -= f.reserved;
       ++completed;
-      inflight[k] = inflight.back();
-      inflight.pop_back();
     }
+    inflight.swap(staying);
     // nothing left to step but events still counted live: inconsistent state
     if (done == 0 && !inflight.empty()) return CELER_ERR_STATE;
   }

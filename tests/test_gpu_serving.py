@@ -124,3 +124,27 @@ def test_consecutive_admissions_track_the_buffer_fill_level():
         for e, ev in ((0, a), (1, b), (2, c)):
             tally, esc = ctx.read_tallies(e)
             assert tally.sum() + esc == pytest.approx(ev["E"].sum(), rel=1e-12)
+
+
+@pytest.mark.parametrize("mode,policy,chunk", [(binding.LOOP_HOST, wl.SORT_LOCAL, 4), (binding.LOOP_ASYNC, wl.SORT_LOCAL, 1),
+                                               (binding.LOOP_ASYNC, wl.SORT_LOCAL, 100_000),
+                                               (binding.LOOP_PERSISTENT, wl.SORT_NONE, 100_000)])
+def test_many_events_end_in_one_chunk(mode, policy, chunk):
+    """More events than tally rows, several ending in the same chunk: each gets
+    its own tallies."""
+    n = 70
+    events = [wl.electron_beam(1 + i % 5, 20.0 + 3.0 * i, event=i) for i in range(n)]
+    prob = wl.calorimeter_problem(1 << 13, max_events=40, sort_policy=policy)
+    with binding.Context(prob) as ctx:
+        res, summ, tallies = ctx.serve([(0.0, i, e) for i, e in enumerate(events)], mode=mode, chunk_iterations=chunk,
+                                       with_tallies=True)
+    assert summ["completed"] == n
+    with binding.Context(prob.replace(max_events=n)) as ctx:
+        for e in events:
+            ctx.add_events(e)
+        ctx.run_events(mode)
+        for i in range(n):
+            want, escaped = ctx.read_tallies(i)
+            np.testing.assert_allclose(tallies[i], want, rtol=1e-12, atol=1e-9)
+            assert res["escaped"][i] == pytest.approx(escaped, rel=1e-12, abs=1e-9)
+            assert res["edep"][i] == pytest.approx(want.sum(), rel=1e-12, abs=1e-9)
