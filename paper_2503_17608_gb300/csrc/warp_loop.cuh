@@ -759,7 +759,11 @@ __device__ __noinline__ void store_tracks(const Params& p, const TrackCache<kCap
   const unsigned n = s_n;
   const unsigned lane = threadIdx.x & 31u, nwarps = blockDim.x >> 5;
   for (uint32_t g = (uint32_t)bid + (uint32_t)nb * (threadIdx.x >> 5); g < p.n_chunks; g += (uint32_t)nb * nwarps) {
-    if (*reinterpret_cast<volatile unsigned*>(&s_next) >= n) break;
+    // (read by lane 0: other warps move it, and the warp leaves as a whole or
+    // not at all)
+    unsigned next = 0;
+    if (lane == 0) next = *reinterpret_cast<volatile unsigned*>(&s_next);
+    if (__shfl_sync(0xffffffffu, next, 0) >= n) break;
     const uint32_t slot = g * 32u + lane;
     const bool vac = slot < p.n_slots && p.trk.status[slot] == VACANT;
     const unsigned bal = __ballot_sync(0xffffffffu, vac);
@@ -774,6 +778,7 @@ __device__ __noinline__ void store_tracks(const Params& p, const TrackCache<kCap
       atomicSub(&p.vacant[g], k);
       atomicSub(&p.tile_vacant[g >> 3], k);
     }
+    __syncwarp();
   }
 }
 
