@@ -67,7 +67,7 @@ __device__ __noinline__ bool wq_wait_poll(const Params& p, volatile unsigned* e,
     __nanosleep(20);
     if ((*e >> 16) == state) return true;
     if (clock64() - t0 > timeout) {
-      atomicExch(p.barrier + 2, 1u);
+      atomicOr(p.barrier + 2, ABORT_WAIT);
       atomicOr(&p.ctl->error, ERR_BARRIER_TIMEOUT);
       return false;
     }
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kTile, 1) k_loop_async(Params p) {
     s_vtot = __ldcg(&p.block_vacant[bid]);
     if (__ldcg(&c->local_blocks) != (unsigned)nb) {  // vacancy counts made for another grid
       atomicOr(&c->error, ERR_VACANCY);
-      atomicExch(abort_word, 1u);
+      atomicOr(abort_word, ABORT_RUN);
     }
   }
   __syncthreads();
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kTile, 1) k_loop_async(Params p) {
       t_seen = now;
     } else if (now - t_seen > kBarrierTimeoutCycles) {
       atomicOr(&c->error, ERR_NO_PROGRESS);
-      atomicExch(abort_word, 1u);
+      atomicOr(abort_word, ABORT_RUN);
     }
   };
   for (;;) {
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kTile, 1) k_loop_async(Params p) {
       ++passes;
       if (passes >= max_passes) {
         atomicOr(&c->error, ERR_ITERATIONS);
-        atomicExch(abort_word, 1u);
+        atomicOr(abort_word, ABORT_RUN);
       }
       if (tot.steps == 0) watchdog();
     }

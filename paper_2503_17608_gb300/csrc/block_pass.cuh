@@ -187,7 +187,7 @@ __device__ __forceinline__ bool wait_generation(const Params& p, unsigned g, lon
     if (*reinterpret_cast<volatile unsigned*>(gen) != g) break;
     if (*reinterpret_cast<volatile unsigned*>(abort_word) != 0u) return false;
     if (clock64() - t0 > timeout) {
-      atomicExch(abort_word, 1u);
+      atomicOr(abort_word, ABORT_WAIT);
       atomicOr(&p.ctl->error, ERR_BARRIER_TIMEOUT);
       return false;
     }

@@ -28,6 +28,13 @@ enum ProcBits : int {
 };
 
 enum PType : uint8_t { GAMMA = 0, ELECTRON = 1, POSITRON = 2 };
+// Bits of the abort word (barrier[2]): a bounded wait gave up, so that every
+// other wait gives up at once; or the run ends early (iteration limit, no
+// progress): no block begins anything new, but the reads and writes under way
+// end as ever, since each waits only for the other side's access of the same
+// entry, and no track is lost.
+enum AbortBits : unsigned { ABORT_WAIT = 1u, ABORT_RUN = 2u };
+
 enum Status : uint8_t { VACANT = 0, ALIVE = 1, DEFERRED = 2 };
 
 // Next action of a track, chosen by the step-limit kernel: the

@@ -92,17 +92,20 @@ __device__ __forceinline__ unsigned ring_lap_code(const Params& p, unsigned long
   return (unsigned)(index >> __popcll(p.ring_mask)) * 2u;
 }
 // Bounded wait of one thread for entry `index` to reach state `code`. After
-// `timeout` cycles (~1 s by default), or if another wait gave up first (abort
-// word), it sets the abort word and ERR_BARRIER_TIMEOUT and returns false.
+// `timeout` cycles (~1 s by default), or if another wait gave up first
+// (ABORT_WAIT), it sets ABORT_WAIT and ERR_BARRIER_TIMEOUT and returns false. A
+// run that ends early otherwise (ABORT_RUN) does not end the wait: a claimed
+// entry that is not read, or a reserved one that is not written, is a track
+// lost.
 __device__ __noinline__ bool ring_wait_poll(const Params& p, const unsigned* st, unsigned code, long long timeout) {
   unsigned* abort_word = p.barrier + 2;
   const long long t0 = clock64();
   for (;;) {
     __nanosleep(32);
     if (ld_acquire_u32(st) == code) return true;
-    if (*reinterpret_cast<volatile unsigned*>(abort_word) != 0u) return false;
+    if ((*reinterpret_cast<volatile unsigned*>(abort_word) & ABORT_WAIT) != 0u) return false;
     if (clock64() - t0 > timeout) {
-      atomicExch(abort_word, 1u);
+      atomicOr(abort_word, ABORT_WAIT);
       atomicOr(&p.ctl->error, ERR_BARRIER_TIMEOUT);
       return false;
     }

@@ -846,7 +846,7 @@ static __device__ __noinline__ bool idle_poll(const Params& p, bool empty, unsig
     t_seen = now;
   } else if (now - t_seen > kBarrierTimeoutCycles) {
     atomicOr(&ctl->error, ERR_NO_PROGRESS);
-    atomicExch(p.barrier + 2, 1u);
+    atomicOr(p.barrier + 2, ABORT_RUN);
     return true;
   }
   return false;
@@ -1045,11 +1045,14 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       if (lane == 0 && atomicCAS(&s_filling, 0u, 1u) == 0u) {
         const unsigned free_now = *reinterpret_cast<volatile unsigned*>(&s_tail[W_FREE]) -
                                   *reinterpret_cast<volatile unsigned*>(&s_head[W_FREE]);
-        if (*reinterpret_cast<volatile unsigned*>(&s_parked) != 0u) {
+        const unsigned aborted = *reinterpret_cast<volatile unsigned*>(abort_word);
+        const long long a = (long long)*reinterpret_cast<volatile unsigned long long*>(&ctl->avail);
+        const long long alive = (long long)*reinterpret_cast<volatile unsigned long long*>(&ctl->alive);
+        if (aborted != 0u) {
+          atomicExch(&s_exit, 1u);  // another block ended the run: take nothing more
+        } else if (*reinterpret_cast<volatile unsigned*>(&s_parked) != 0u) {
           load_chunk = next_parked_chunk(p, &s_cursor, &s_parked, bid, nb, n_own, free_now, &take);
         } else {
-          const long long a = (long long)*reinterpret_cast<volatile unsigned long long*>(&ctl->avail);
-          const long long alive = (long long)*reinterpret_cast<volatile unsigned long long*>(&ctl->alive);
           const unsigned live = *reinterpret_cast<volatile unsigned*>(&s_live);
           *reinterpret_cast<volatile unsigned*>(&s_looked) = (unsigned)clock64();
           if (full_buffer && a < (long long)(p.ring_capacity - p.ring_capacity / 8u))
@@ -1092,7 +1095,8 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     unsigned c = kNoEntry;
     int out = W_NONE;
     unsigned n = 0;
-    bool fresh = false;  // the lane's track needs a number of mean free paths
+    bool fresh = false;    // the lane's track needs a number of mean free paths
+    bool gave_up = false;  // the lane's wait in a fill gave up
     unsigned meta = 0;
     TrackRng rng(p.seed, 0u, 0ull, 0u);
     if (take > 0) {
@@ -1105,7 +1109,10 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
         const unsigned bal = __ballot_sync(0xffffffffu, live);
         if (live) {
           c = pop_entry(p, tc, W_FREE, f0 + (unsigned)__popc(bal & lt));
-          if (c != kNoEntry) out = load_entry(p, tc, slot, c);
+          if (c != kNoEntry)
+            out = load_entry(p, tc, slot, c);
+          else
+            gave_up = true;
         }
         // (they were counted alive already)
       } else {
@@ -1132,6 +1139,8 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
             rng = TrackRng(p.seed, r.m.x, tid, 0u);
             fresh = true;
             out = r.m.w == GAMMA ? W_PHOTON : W_ELECTRON;
+          } else {
+            gave_up = true;
           }
         }
       }
@@ -1183,9 +1192,22 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     if (take > 0 || n > 0) {
       if (fresh) renew(p, tc, c, meta, rng);
       __syncwarp();
+      // A fill's waits give up only if the protocol is broken: what was claimed
+      // is lost to the run, which ends with its error status, and the entry is
+      // free again (it never held a track).
+      const unsigned lost = __ballot_sync(0xffffffffu, gave_up);
+      if (lost) {
+        const unsigned back = __ballot_sync(0xffffffffu, gave_up && c != kNoEntry);
+        if (back) push_lanes(p, tc, s_tail, W_FREE, back, c);
+        if (load_chunk == 0xFFFFFFFFu) fill -= (unsigned)__popc(lost);
+        if (lane == 0) {
+          atomicSub(&s_live, (unsigned)__popc(lost));
+          atomicExch(&s_exit, 1u);
+        }
+      }
       // a track whose interaction found no buffer space waits in its queue
       // (draining: in its entry, to be stored deferred)
-      const bool waits = c != kNoEntry && out == W_NONE;
+      const bool waits = !gave_up && c != kNoEntry && out == W_NONE;
       const bool deferred = __any_sync(0xffffffffu, waits);
       if (deferred && lane == 0) *reinterpret_cast<volatile unsigned*>(&s_deferred) = 1u;
       if (waits && !drain) out = (int)pick_k;
@@ -1242,7 +1264,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       if (pieces >= budget && lane == 0) atomicExch(&s_drain, 1u);
       if (pieces >= max_pieces && lane == 0) {
         atomicOr(&ctl->error, ERR_ITERATIONS);
-        atomicExch(abort_word, 1u);
+        atomicOr(abort_word, ABORT_RUN);
         atomicExch(&s_exit, 1u);
       }
       // a piece without deferrals made progress; one with deferrals (the
