@@ -35,7 +35,10 @@ enum PType : uint8_t { GAMMA = 0, ELECTRON = 1, POSITRON = 2 };
 // entry, and no track is lost.
 enum AbortBits : unsigned { ABORT_WAIT = 1u, ABORT_RUN = 2u };
 
-enum Status : uint8_t { VACANT = 0, ALIVE = 1, DEFERRED = 2 };
+// In k_loop_warps only (no slot is left so at the end of a run): HELD, the
+// slot's track is in its block's shared memory; CLAIMED beside ALIVE or
+// DEFERRED, a warp is about to load it.
+enum Status : uint8_t { VACANT = 0, ALIVE = 1, DEFERRED = 2, HELD = 3, CLAIMED = 4 };
 
 // Next action of a track, chosen by the step-limit kernel: the
 // geometric/range limits handled by the along-step kernels, then the

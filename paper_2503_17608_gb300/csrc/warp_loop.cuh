@@ -661,7 +661,7 @@ __device__ __forceinline__ void renew(const Params& p, const TrackCache<kCap>& t
 template <int kCap>
 __device__ __noinline__ int load_entry(const Params& p, const TrackCache<kCap>& tc, uint32_t slot, unsigned c) {
   const Tracks& t = p.trk;
-  const uint8_t st = t.status[slot], pt = t.ptype[slot];
+  const uint8_t st = t.status[slot] & 3u, pt = t.ptype[slot];
   const double nmfp = t.nmfp[slot];
   tc.x(c) = t.x[slot];
   tc.y(c) = t.y[slot];
@@ -677,6 +677,7 @@ __device__ __noinline__ int load_entry(const Params& p, const TrackCache<kCap>& 
   tc.event(c) = t.event[slot];
   tc.primary(c) = t.primary[slot];
   tc.home(c) = slot;
+  t.status[slot] = HELD;
   const bool pending = st == DEFERRED;
   const uint8_t act = pending ? t.action[slot] : (uint8_t)A_NONE;
   const unsigned meta = kMetaLive | kMetaStored | ((unsigned)act << 26) | ((unsigned)pt << 24) |
@@ -716,26 +717,70 @@ __device__ __forceinline__ void store_entry(const Params& p, const TrackCache<kC
   t.status[slot] = meta_act(meta) != 0 ? DEFERRED : ALIVE;
 }
 
-// The next chunk with parked tracks, if `free_now` entries suffice for it: its
-// index (or ~0), its live tracks in *take, the cursor and the count of parked
-// tracks moved on (one thread, under the block's fill lock).
-static __device__ __noinline__ uint32_t next_parked_chunk(const Params& p, unsigned* s_cursor, unsigned* s_parked, int bid,
-                                                          int nb, uint32_t n_own, unsigned free_now, unsigned* take) {
-  volatile unsigned* cursor = s_cursor;
-  while (*cursor < n_own) {
-    const uint32_t g = (uint32_t)bid + (uint32_t)nb * *cursor;
-    unsigned cnt = 0;
-#pragma unroll 1
-    for (uint32_t s = g * 32u; s < g * 32u + 32u && s < p.n_slots; ++s) cnt += p.trk.status[s] != VACANT ? 1u : 0u;
+// Slots of block bid.
+__device__ __forceinline__ unsigned owned_slots(const Params& p, int bid, int nb, uint32_t n_own) {
+  const bool owns_last = n_own > 0 && (uint32_t)bid + (uint32_t)nb * (n_own - 1u) == p.n_chunks - 1u;
+  return n_own * 32u - (owns_last ? p.n_chunks * 32u - p.n_slots : 0u);
+}
+
+// A block's control words in shared memory that the functions below move too:
+// one address for all of them, so that the loop keeps none of them in registers
+// for the calls.
+struct BlockWords {
+  unsigned head[kWarpKinds + 1], tail[kWarpKinds + 1];  // of the queues
+  unsigned live, parked, cursor, filling, exit, place;
+};
+__device__ __forceinline__ unsigned block_word(const unsigned& a) { return *reinterpret_cast<const volatile unsigned*>(&a); }
+
+// The next chunk with parked tracks, if as many entries are free: its index (or
+// ~0), its parked tracks in `take`, the first of the free entries claimed for
+// them in f0. While the buffer is full (moving_only) the tracks whose
+// interactions wait for room in it stay where they are. The tracks are marked,
+// so that the warp can load them without the block's fill lock, which lane 0
+// holds and this gives up. The whole warp calls it. (One lane looking at the
+// chunk's slots in turn: a run that starts with 140,000 tracks, 0.9 -> 2.0 ms.)
+static __device__ __noinline__ uint32_t claim_parked_chunk(const Params& p, BlockWords& w, int bid, int nb, uint32_t n_own,
+                                                           bool moving_only, unsigned& take, unsigned& f0) {
+  const unsigned lane = threadIdx.x & 31u;
+  unsigned m = 0, free_now = 0;
+  if (lane == 0) {
+    m = block_word(w.cursor);
+    free_now = block_word(w.tail[W_FREE]) - block_word(w.head[W_FREE]);
+  }
+  m = __shfl_sync(0xffffffffu, m, 0);
+  free_now = __shfl_sync(0xffffffffu, free_now, 0);
+  uint32_t g = 0xFFFFFFFFu;
+  unsigned next = m;  // no parked track waits in a chunk before it
+  take = 0;
+  for (; m < n_own; ++m) {
+    const uint32_t at = (uint32_t)bid + (uint32_t)nb * m, slot = at * 32u + lane;
+    volatile uint8_t* status = p.trk.status + slot;
+    const uint8_t st = slot < p.n_slots ? *status : (uint8_t)VACANT;
+    const bool parked = st == ALIVE || (st == DEFERRED && !moving_only);
+    const unsigned cnt = (unsigned)__popc(__ballot_sync(0xffffffffu, parked));
+    const bool left = __any_sync(0xffffffffu, st == DEFERRED && moving_only);
     if (cnt > free_now) break;
-    *cursor = *cursor + 1u;
+    if (next == m && !left) next = m + 1u;
     if (cnt > 0) {
-      *take = cnt;
-      atomicSub(s_parked, cnt);
-      return g;
+      if (parked) *status = st | CLAIMED;
+      take = cnt;
+      g = at;
+      break;
     }
   }
-  return 0xFFFFFFFFu;
+  f0 = 0;
+  if (lane == 0) {
+    *reinterpret_cast<volatile unsigned*>(&w.cursor) = next;
+    if (take) {
+      f0 = atomicAdd(&w.head[W_FREE], take);  // only the holder of the lock claims free entries
+      atomicAdd(&w.live, take);
+      atomicSub(&w.parked, take);
+    }
+  }
+  __threadfence_block();
+  __syncwarp();
+  if (lane == 0) atomicExch(&w.filling, 0u);
+  return g;
 }
 
 // The tracks still live at the end of a run back into the block's slots:
@@ -780,6 +825,113 @@ __device__ __noinline__ void store_tracks(const Params& p, const TrackCache<kCap
     }
     __syncwarp();
   }
+}
+
+// A block whose every entry holds a track that waits for buffer space moves up
+// to 32 of them into its slots (their own, or vacant ones), their interactions
+// pending, as the end of a run would store them; the entries take tracks out of
+// the buffer then, which makes room in it, or parked tracks that can move.
+// claim_parked_chunk brings them back once there is room. Not where nothing
+// could take the entries: the block has no slot to spare and no track parked.
+// (Without it a block could hold no more tracks than entries: 6 materials, 256
+// entries, 20,000 x 1 GeV with a buffer of 2^17 ended with every entry of every
+// block waiting.) The whole warp calls it.
+template <int kCap>
+__device__ __noinline__ void park_waiting(const Params& p, const TrackCache<kCap>& tc, BlockWords& w, int bid, int nb,
+                                          uint32_t n_own) {
+  const unsigned lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+  bool mine = false;
+  uint32_t g = 0xFFFFFFFFu;  // a chunk with vacant slots
+  unsigned h = 0, n = 0;
+  int k = W_PAIR;
+  if (lane == 0 && atomicCAS(&w.filling, 0u, 1u) == 0u) {
+    mine = true;
+    const unsigned parked = block_word(w.parked);
+    if (block_word(w.tail[W_FREE]) == block_word(w.head[W_FREE]) &&
+        (parked != 0u || block_word(w.live) < owned_slots(p, bid, nb, n_own))) {
+      unsigned m = block_word(w.place);
+      for (uint32_t i = 0; i < n_own && g == 0xFFFFFFFFu; ++i) {
+        if (__ldcg(&p.vacant[(uint32_t)bid + (uint32_t)nb * m]) != 0u)
+          g = (uint32_t)bid + (uint32_t)nb * m;
+        else
+          m = m + 1u < n_own ? m + 1u : 0u;
+      }
+      *reinterpret_cast<volatile unsigned*>(&w.place) = m;
+      unsigned most = 0;
+      for (int j = W_PAIR; j <= W_BREMS; ++j) {
+        const unsigned hd = block_word(w.head[j]), q = block_word(w.tail[j]) - hd;  // the head before the tail
+        if (q > most) {
+          most = q;
+          k = j;
+          h = hd;
+        }
+      }
+      n = min(most, 32u);
+      if (n && atomicCAS(&w.head[k], h, h + n) != h) n = 0;  // another warp claimed: next time
+    }
+  }
+  n = __shfl_sync(0xffffffffu, n, 0);
+  if (n) {
+    g = __shfl_sync(0xffffffffu, g, 0);
+    h = __shfl_sync(0xffffffffu, h, 0);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    const uint32_t slot0 = g * 32u + lane;
+    const bool vac = g != 0xFFFFFFFFu && slot0 < p.n_slots &&
+                     *reinterpret_cast<volatile uint8_t*>(p.trk.status + slot0) == VACANT;
+    const unsigned bal = __ballot_sync(0xffffffffu, vac);
+    const unsigned c = lane < n ? pop_entry(p, tc, k, h + lane) : kNoEntry;
+    const bool stored = c != kNoEntry && (tc.meta(c) & kMetaStored) != 0u;
+    const unsigned rank = (unsigned)__popc(__ballot_sync(0xffffffffu, c != kNoEntry && !stored) & lt);
+    const bool placed = c != kNoEntry && !stored && rank < (unsigned)__popc(bal);
+    const unsigned new_mask = __ballot_sync(0xffffffffu, placed), all = __ballot_sync(0xffffffffu, stored || placed);
+    const unsigned rest = __ballot_sync(0xffffffffu, c != kNoEntry && !stored && !placed);
+    if (stored || placed) {
+      uint32_t slot = tc.home(c);
+      if (placed) {  // the vacant slot of its rank
+        unsigned left = bal;
+        for (unsigned r = rank; r > 0; --r) left &= left - 1u;
+        slot = g * 32u + (unsigned)(__ffs(left) - 1);
+      }
+      store_entry(p, tc, slot, c);
+      tc.meta(c) = 0u;
+      atomicMin(&w.cursor, ((slot >> 5) - (uint32_t)bid) / (uint32_t)nb);
+    }
+    if (lane == 0 && new_mask) {
+      atomicSub(&p.vacant[g], (unsigned)__popc(new_mask));
+      atomicSub(&p.tile_vacant[g >> 3], (unsigned)__popc(new_mask));
+    }
+    if (rest) push_lanes(p, tc, w.tail, k, rest, c);
+    if (all) {
+      push_lanes(p, tc, w.tail, W_FREE, all, c);
+      if (lane == 0) {
+        atomicAdd(&w.parked, (unsigned)__popc(all));
+        atomicSub(&w.live, (unsigned)__popc(all));
+      }
+    }
+    __syncwarp();
+  }
+  if (mine) {
+    __threadfence_block();
+    atomicExch(&w.filling, 0u);
+  }
+  __syncwarp();
+}
+
+// A fill's wait gives up only if the buffer's protocol is broken: what the lanes
+// had claimed is lost to the run, which ends with its error status, and their
+// entries, which never held a track, are free again. The whole warp calls it;
+// returns how many lanes gave up.
+template <int kCap>
+__device__ __noinline__ unsigned give_back(const Params& p, const TrackCache<kCap>& tc, BlockWords& w, bool gave_up,
+                                           unsigned c) {
+  const unsigned lost = (unsigned)__popc(__ballot_sync(0xffffffffu, gave_up));
+  const unsigned back = __ballot_sync(0xffffffffu, gave_up && c != kNoEntry);
+  if (back) push_lanes(p, tc, w.tail, W_FREE, back, c);
+  if ((threadIdx.x & 31u) == 0u) {
+    atomicSub(&w.live, lost);
+    atomicExch(&w.exit, 1u);
+  }
+  return lost;
 }
 
 // Warps of a block that take pieces of any size; the others take full pieces
@@ -865,14 +1017,15 @@ static __device__ __noinline__ bool idle_poll(const Params& p, bool empty, unsig
 // progress) does the same, without the interactions that need the buffer. A
 // block that starts with more live tracks than it has entries steps them in
 // turns: `parked` of them wait in their slots, and entries that come free take
-// them, before any initializer.
+// them, before any initializer unless the buffer is full. A block that runs out
+// of entries while the buffer is full parks tracks too (park_waiting).
 template <int kCap>
 __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TrackCache<kCap> tc{smem_raw};
   const SharedStatic ss = carve_static(p, smem_raw + TrackCache<kCap>::kBytes);
-  __shared__ unsigned s_head[kWarpKinds + 1], s_tail[kWarpKinds + 1];
-  __shared__ unsigned s_live, s_filling, s_exit, s_drain, s_parked, s_cursor, s_kind, s_looked, s_deferred;
+  __shared__ BlockWords w;
+  __shared__ unsigned s_drain, s_kind, s_looked, s_deferred;
   __shared__ unsigned s_vacant;
   __shared__ unsigned long long s_pieces;
   const int nb = (int)gridDim.x, bid = (int)blockIdx.x;
@@ -881,8 +1034,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   Ctl* ctl = p.ctl;
   unsigned* abort_word = p.barrier + 2;
   const uint32_t n_own = (uint32_t)bid < p.n_chunks ? (p.n_chunks - (uint32_t)bid + nb - 1) / nb : 0u;
-  const bool owns_last = n_own > 0 && (uint32_t)bid + (uint32_t)nb * (n_own - 1u) == p.n_chunks - 1u;
-  const unsigned owned = n_own * 32u - (owns_last ? p.n_chunks * 32u - p.n_slots : 0u);
+  const unsigned owned = owned_slots(p, bid, nb, n_own);
   const unsigned n_entries = owned < (unsigned)kCap ? owned : (unsigned)kCap;
   const unsigned long long max_pieces = __ldcg(&ctl->max_iterations);  // per run
   const unsigned long long budget = p.run_budget;
@@ -900,19 +1052,20 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     *tc.queue(W_FREE, c) = c < n_entries ? ((1u << 16) | c) : 0u;  // every entry free, lap 0 written
   }
   if (threadIdx.x <= kWarpKinds) {
-    s_head[threadIdx.x] = 0u;
-    s_tail[threadIdx.x] = threadIdx.x == W_FREE ? n_entries : 0u;
+    w.head[threadIdx.x] = 0u;
+    w.tail[threadIdx.x] = threadIdx.x == W_FREE ? n_entries : 0u;
   }
   if (threadIdx.x == 0) {
-    s_live = 0u;
-    s_filling = 0u;
-    s_exit = 0u;
+    w.live = 0u;
+    w.filling = 0u;
+    w.exit = 0u;
     s_drain = 0u;
     s_pieces = 0ull;
-    s_cursor = 0u;
-    s_parked = 0u;
+    w.cursor = 0u;
+    w.parked = 0u;
     s_kind = (unsigned)W_PHOTON;
     s_deferred = 0u;
+    w.place = 0u;
     s_looked = (unsigned)clock64() - 2u * kLookCycles;
   }
   double* thick = reinterpret_cast<double*>(smem_raw + TrackCache<kCap>::kBytes + p.static_bytes);  // layer thicknesses
@@ -921,7 +1074,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   const unsigned live0 = owned - s_vacant;
   if (threadIdx.x == 0) {
     atomicAdd(&ctl->vacant_seen, (unsigned long long)s_vacant);
-    if (live0 > n_entries) s_parked = live0;  // they wait in their slots until entries take them
+    if (live0 > n_entries) w.parked = live0;  // they wait in their slots until entries take them
   }
   if (live0 > 0 && live0 <= n_entries) {
     // the live tracks of the block's chunks, one chunk per warp at a time,
@@ -932,7 +1085,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       const unsigned bal = __ballot_sync(0xffffffffu, live);
       if (bal == 0u) continue;
       unsigned f = 0;
-      if (lane == 0) f = atomicAdd(&s_head[W_FREE], (unsigned)__popc(bal));
+      if (lane == 0) f = atomicAdd(&w.head[W_FREE], (unsigned)__popc(bal));
       f = __shfl_sync(0xffffffffu, f, 0) + (unsigned)__popc(bal & lt);
       unsigned c = kNoEntry;
       int k = W_NONE;
@@ -943,11 +1096,11 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       for (unsigned todo = __ballot_sync(0xffffffffu, k != W_NONE); todo;) {
         const int kk = __shfl_sync(0xffffffffu, k, __ffs(todo) - 1);
         const unsigned m2 = __ballot_sync(0xffffffffu, k == kk);
-        push_lanes(p, tc, s_tail, kk, m2, c);
+        push_lanes(p, tc, w.tail, kk, m2, c);
         todo &= ~m2;
       }
     }
-    if (threadIdx.x == 0) s_live = live0;
+    if (threadIdx.x == 0) w.live = live0;
   }
   __syncthreads();
   unsigned steps = 0, killed = 0, fill = 0, events = 0;
@@ -965,9 +1118,9 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     // diverged, and a lane leaving alone would strand the others' shuffles)
     unsigned flags = 0;
     if (lane == 0)
-      flags = (*reinterpret_cast<volatile unsigned*>(&s_exit) != 0u ? 1u : 0u) |
+      flags = (*reinterpret_cast<volatile unsigned*>(&w.exit) != 0u ? 1u : 0u) |
               (*reinterpret_cast<volatile unsigned*>(&s_drain) != 0u ? 2u : 0u) |
-              (*reinterpret_cast<volatile unsigned*>(&s_live) >= kManyLive ? 4u : 0u) |
+              (*reinterpret_cast<volatile unsigned*>(&w.live) >= kManyLive ? 4u : 0u) |
               (*reinterpret_cast<volatile unsigned*>(&s_deferred) != 0u ? 8u : 0u);
     flags = __shfl_sync(0xffffffffu, flags, 0);
     const bool drain = (flags & 3u) != 0u, many = (flags & 4u) != 0u, full_buffer = (flags & 8u) != 0u;
@@ -989,8 +1142,8 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     // spread over many part-filled ones.
     unsigned waiting = 0;
     if (lane < kWarpKinds && ((allowed >> lane) & 1u)) {
-      const unsigned hd = *reinterpret_cast<volatile unsigned*>(&s_head[lane]);  // before the tail: hd <= tail
-      waiting = *reinterpret_cast<volatile unsigned*>(&s_tail[lane]) - hd;
+      const unsigned hd = *reinterpret_cast<volatile unsigned*>(&w.head[lane]);  // before the tail: hd <= tail
+      waiting = *reinterpret_cast<volatile unsigned*>(&w.tail[lane]) - hd;
     }
     constexpr unsigned kMovingKinds = (1u << W_PHOTON) | (1u << W_ELECTRON) | (1u << W_COMPTON);  // make no tracks
     constexpr unsigned kChargedKinds = (1u << W_ELECTRON) | (1u << W_MOLLER) | (1u << W_BREMS);
@@ -1036,27 +1189,32 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     unsigned take = 0, f0 = 0;
     unsigned long long first = 0;
     uint32_t load_chunk = 0xFFFFFFFFu;  // a chunk of parked tracks to load
+    constexpr unsigned kParked = 0xFFFFFFFFu;
     // (interactions wait for buffer space: entries must be taken whatever the
     // target, or no block would make room for another)
+    if (full_buffer && !drain && !helper && (some & kMovingKinds) == 0u)
+      park_waiting(p, tc, w, bid, nb, n_own);
     bool look = !drain && !helper && (scarce || full_buffer);
     if (look && some != 0u)  // work waits here: look at the buffer every kLookCycles at most
       look = (unsigned)clock64() - *reinterpret_cast<volatile unsigned*>(&s_looked) > kLookCycles;
     if (__any_sync(0xffffffffu, look)) {
-      if (lane == 0 && atomicCAS(&s_filling, 0u, 1u) == 0u) {
-        const unsigned free_now = *reinterpret_cast<volatile unsigned*>(&s_tail[W_FREE]) -
-                                  *reinterpret_cast<volatile unsigned*>(&s_head[W_FREE]);
-        const unsigned aborted = *reinterpret_cast<volatile unsigned*>(abort_word);
+      if (lane == 0 && atomicCAS(&w.filling, 0u, 1u) == 0u) {
+        const unsigned free_now = *reinterpret_cast<volatile unsigned*>(&w.tail[W_FREE]) -
+                                  *reinterpret_cast<volatile unsigned*>(&w.head[W_FREE]);
         const long long a = (long long)*reinterpret_cast<volatile unsigned long long*>(&ctl->avail);
         const long long alive = (long long)*reinterpret_cast<volatile unsigned long long*>(&ctl->alive);
-        if (aborted != 0u) {
-          atomicExch(&s_exit, 1u);  // another block ended the run: take nothing more
-        } else if (*reinterpret_cast<volatile unsigned*>(&s_parked) != 0u) {
-          load_chunk = next_parked_chunk(p, &s_cursor, &s_parked, bid, nb, n_own, free_now, &take);
+        const unsigned live = *reinterpret_cast<volatile unsigned*>(&w.live);
+        const unsigned parked = *reinterpret_cast<volatile unsigned*>(&w.parked);
+        if (full_buffer && a < (long long)(p.ring_capacity - p.ring_capacity / 8u))
+          *reinterpret_cast<volatile unsigned*>(&s_deferred) = 0u;  // an eighth of it is free again
+        // parked tracks come before initializers, unless the buffer is full:
+        // then as many of those as the block has slots for
+        unsigned spare = 0u;
+        if (parked != 0u && full_buffer && a > 0) spare = owned_slots(p, bid, nb, n_own) - live - parked;
+        if (parked != 0u && spare == 0u) {
+          take = kParked;  // (the lock stays held)
         } else {
-          const unsigned live = *reinterpret_cast<volatile unsigned*>(&s_live);
           *reinterpret_cast<volatile unsigned*>(&s_looked) = (unsigned)clock64();
-          if (full_buffer && a < (long long)(p.ring_capacity - p.ring_capacity / 8u))
-            *reinterpret_cast<volatile unsigned*>(&s_deferred) = 0u;  // an eighth of it is free again
           if (a > 0 && free_now > 0) {
             // at least this block's part of the buffer's entries, and up to
             // its target (single precision does for both)
@@ -1066,6 +1224,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
             unsigned want = (unsigned)fminf(more, 32.0f);
             if (want > free_now) want = free_now;
             if ((long long)want > a) want = (unsigned)a;
+            if (parked != 0u && want > spare) want = spare;
             if (want > 0u) {
               const long long old = (long long)atomicAdd(&ctl->avail, 0ull - (unsigned long long)want);
               if (old >= (long long)want) {
@@ -1083,20 +1242,22 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
             if (a <= 0 || n_entries == 0u) atomicExch(&s_drain, 1u);
           }
         }
-        if (take > 0) {
-          f0 = atomicAdd(&s_head[W_FREE], take);  // only the filler claims free entries
-          atomicAdd(&s_live, take);
+        if (take != kParked) {
+          if (take > 0) {
+            f0 = atomicAdd(&w.head[W_FREE], take);  // only the filler claims free entries
+            atomicAdd(&w.live, take);
+          }
+          __threadfence_block();
+          atomicExch(&w.filling, 0u);
         }
-        __threadfence_block();
-        atomicExch(&s_filling, 0u);
       }
       take = __shfl_sync(0xffffffffu, take, 0);
+      if (take == kParked) load_chunk = claim_parked_chunk(p, w, bid, nb, n_own, full_buffer, take, f0);
     }
     unsigned c = kNoEntry;
     int out = W_NONE;
     unsigned n = 0;
-    bool fresh = false;    // the lane's track needs a number of mean free paths
-    bool gave_up = false;  // the lane's wait in a fill gave up
+    bool fresh = false;  // the lane's track needs a number of mean free paths
     unsigned meta = 0;
     TrackRng rng(p.seed, 0u, 0ull, 0u);
     if (take > 0) {
@@ -1105,14 +1266,13 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       load_chunk = __shfl_sync(0xffffffffu, load_chunk, 0);
       if (load_chunk != 0xFFFFFFFFu) {
         const uint32_t slot = load_chunk * 32u + (uint32_t)lane;
-        const bool live = slot < p.n_slots && p.trk.status[slot] != VACANT;
+        __threadfence_block();
+        const bool live =
+            slot < p.n_slots && (*reinterpret_cast<volatile uint8_t*>(p.trk.status + slot) & CLAIMED) != 0u;
         const unsigned bal = __ballot_sync(0xffffffffu, live);
         if (live) {
           c = pop_entry(p, tc, W_FREE, f0 + (unsigned)__popc(bal & lt));
-          if (c != kNoEntry)
-            out = load_entry(p, tc, slot, c);
-          else
-            gave_up = true;
+          if (c != kNoEntry) out = load_entry(p, tc, slot, c);
         }
         // (they were counted alive already)
       } else {
@@ -1139,9 +1299,11 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
             rng = TrackRng(p.seed, r.m.x, tid, 0u);
             fresh = true;
             out = r.m.w == GAMMA ? W_PHOTON : W_ELECTRON;
-          } else {
-            gave_up = true;
           }
+        }
+        if (__any_sync(0xffffffffu, (unsigned)lane < take && out == W_NONE)) {
+          fill -= give_back(p, tc, w, (unsigned)lane < take && out == W_NONE, c);
+          if (out == W_NONE) c = kNoEntry;
         }
       }
     } else if (pick_k != 0xFFu) {
@@ -1149,11 +1311,11 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       unsigned h = 0;
       if (lane == 0) {
         for (int a = 0; a < 8; ++a) {
-          h = *reinterpret_cast<volatile unsigned*>(&s_head[pick_k]);
-          const unsigned q = *reinterpret_cast<volatile unsigned*>(&s_tail[pick_k]) - h;
+          h = *reinterpret_cast<volatile unsigned*>(&w.head[pick_k]);
+          const unsigned q = *reinterpret_cast<volatile unsigned*>(&w.tail[pick_k]) - h;
           if (q == 0) break;
           const unsigned want = q < 32u ? q : 32u;
-          if (atomicCAS(&s_head[pick_k], h, h + want) == h) {
+          if (atomicCAS(&w.head[pick_k], h, h + want) == h) {
             n = want;
             break;
           }
@@ -1192,22 +1354,9 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     if (take > 0 || n > 0) {
       if (fresh) renew(p, tc, c, meta, rng);
       __syncwarp();
-      // A fill's waits give up only if the protocol is broken: what was claimed
-      // is lost to the run, which ends with its error status, and the entry is
-      // free again (it never held a track).
-      const unsigned lost = __ballot_sync(0xffffffffu, gave_up);
-      if (lost) {
-        const unsigned back = __ballot_sync(0xffffffffu, gave_up && c != kNoEntry);
-        if (back) push_lanes(p, tc, s_tail, W_FREE, back, c);
-        if (load_chunk == 0xFFFFFFFFu) fill -= (unsigned)__popc(lost);
-        if (lane == 0) {
-          atomicSub(&s_live, (unsigned)__popc(lost));
-          atomicExch(&s_exit, 1u);
-        }
-      }
       // a track whose interaction found no buffer space waits in its queue
       // (draining: in its entry, to be stored deferred)
-      const bool waits = !gave_up && c != kNoEntry && out == W_NONE;
+      const bool waits = c != kNoEntry && out == W_NONE;
       const bool deferred = __any_sync(0xffffffffu, waits);
       if (deferred && lane == 0) *reinterpret_cast<volatile unsigned*>(&s_deferred) = 1u;
       if (waits && !drain) out = (int)pick_k;
@@ -1227,12 +1376,12 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
       }
       if (ended) {
         killed += (unsigned)__popc(ended);
-        if (lane == 0) atomicSub(&s_live, (unsigned)__popc(ended));
+        if (lane == 0) atomicSub(&w.live, (unsigned)__popc(ended));
       }
       for (unsigned todo = __ballot_sync(0xffffffffu, out != W_NONE); todo;) {
         const int kk = __shfl_sync(0xffffffffu, out, __ffs(todo) - 1);
         const unsigned m2 = __ballot_sync(0xffffffffu, out == kk);
-        push_lanes(p, tc, s_tail, kk, m2, c);
+        push_lanes(p, tc, w.tail, kk, m2, c);
         todo &= ~m2;
       }
 #ifdef CELER_LANE_COUNTERS
@@ -1258,14 +1407,19 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
         }
       }
 #endif
-      if ((++events & 15u) == 0) flush_warp_counts(p, steps, killed, fill);  // and whenever the warp idles
+      if ((++events & 15u) == 0) {  // and whenever the warp idles
+        flush_warp_counts(p, steps, killed, fill);
+        // (a warp that never idles sees here that another block ended the run)
+        if ((events & 63u) == 0 && lane == 0 && *reinterpret_cast<volatile unsigned*>(abort_word) != 0u)
+          atomicExch(&w.exit, 1u);
+      }
       if (take > 0) continue;
       ++pieces;
       if (pieces >= budget && lane == 0) atomicExch(&s_drain, 1u);
       if (pieces >= max_pieces && lane == 0) {
         atomicOr(&ctl->error, ERR_ITERATIONS);
         atomicOr(abort_word, ABORT_RUN);
-        atomicExch(&s_exit, 1u);
+        atomicExch(&w.exit, 1u);
       }
       // a piece without deferrals made progress; one with deferrals (the
       // buffer is full) goes on to the idle path: watchdog and a pause
@@ -1274,9 +1428,9 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     // nothing done: leave if every track has ended, else poll (bounded)
     flush_warp_counts(p, steps, killed, fill);
     if (lane == 0) {
-      const bool empty = *reinterpret_cast<volatile unsigned*>(&s_live) == 0u &&
-                         *reinterpret_cast<volatile unsigned*>(&s_parked) == 0u;
-      if (idle_poll(p, empty && budget == ~0ull, seen, t_seen)) atomicExch(&s_exit, 1u);
+      const bool empty = *reinterpret_cast<volatile unsigned*>(&w.live) == 0u &&
+                         *reinterpret_cast<volatile unsigned*>(&w.parked) == 0u;
+      if (idle_poll(p, empty && budget == ~0ull, seen, t_seen)) atomicExch(&w.exit, 1u);
       __nanosleep(500);
 #ifdef CELER_LANE_COUNTERS
       lane_site_n(LS_IDLE, 0u);
@@ -1288,7 +1442,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
   flush_warp_counts(p, steps, killed, fill);
   if (lane == 0) atomicMax(&s_pieces, pieces);
   __syncthreads();
-  const unsigned live = s_live;
+  const unsigned live = w.live;
   if (live > 0)
     store_tracks(p, tc, reinterpret_cast<uint16_t*>(const_cast<unsigned*>(tc.queue(0, 0u))), n_entries, bid, nb);
   if (threadIdx.x == 0) end_async_block(p, nb, s_pieces);
