@@ -353,8 +353,9 @@ celer_status celer_set_parent_reuse(celer_ctx* ctx, int on);
  * two warps of a block take only full pieces of 32, and all of them while the
  * block holds many tracks (budgeted runs, such as a serving loop's chunks, let
  * every warp take any piece otherwise). A block keeps its
- * live tracks in shared memory, at most 1024 of them (256 with more than four
- * materials); a block that starts a run with more steps them in turns.
+ * live tracks in shared memory, as many as fit beside the tables (1024 with up
+ * to five materials and some hundred layers, 512 up to eight, 256 with several
+ * hundred layers of those); a block that has more steps them in turns.
  * Histories do not change. On by default. Takes effect at the next run. on outside
  * {0, 1}: CELER_ERR_INVALID. */
 celer_status celer_set_async_warps(celer_ctx* ctx, int on);

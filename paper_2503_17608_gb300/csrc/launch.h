@@ -29,7 +29,7 @@ struct LaunchShape {
   int block;           // threads per block of the step / along-step / interaction kernels
   size_t static_smem;  // tables + layer planes + layer materials in shared memory
   size_t warp_smem;    // the per-warp schedule: the block's tracks beside them
-  bool warp_small;     // its variant with fewer tracks per block
+  int warp_variant;    // its variant (tracks per block)
 };
 
 cudaError_t configure_kernels(const Params& p, int block, LaunchShape* shape);

@@ -1969,6 +1969,22 @@ __global__ void k_copy_out(uint32_t* dst, const uint32_t* src, uint32_t n, uint3
   for (uint32_t i = first; i < n2; i += stride) dst2[i] = __ldcg(src2 + i);
 }
 
+// The per-warp schedule's kernels by tracks per block, and the bytes of those.
+constexpr int kWarpVariants = 3;
+struct WarpKernel {
+  const void* fn;
+  size_t bytes;
+  int threads;
+};
+template <int kCap>
+WarpKernel warp_kernel_of() {
+  return WarpKernel{(const void*)k_loop_warps<kCap>, TrackCache<kCap>::kBytes, kThreads<kCap>};
+}
+WarpKernel warp_kernel(int variant) {
+  return variant == 0 ? warp_kernel_of<kWarpTracks>()
+                      : (variant == 1 ? warp_kernel_of<kWarpTracksMid>() : warp_kernel_of<kWarpTracksSmall>());
+}
+
 int occupancy_grid(const void* fn, int block, size_t smem, int sms, int cap) {
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem) != cudaSuccess || nb < 1) nb = 1;
@@ -1996,16 +2012,18 @@ cudaError_t configure_kernels(const Params& p, int block, LaunchShape* sh) {
     if (e != cudaSuccess) return e;
   }
   // the per-warp schedule keeps a block's tracks in shared memory: as many as
-  // fit beside the static tables (1,024 up to four materials, else 256)
+  // fit beside the static tables
   int max_smem = 0;
   e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  cudaFuncAttributes fa{};
-  e = cudaFuncGetAttributes(&fa, (const void*)k_loop_warps<kWarpTracks>);
-  if (e != cudaSuccess) return e;
-  sh->warp_small = fa.sharedSizeBytes + TrackCache<kWarpTracks>::kBytes + stat + (size_t)p.n_layers * sizeof(double) > (size_t)max_smem;
-  sh->warp_smem = stat + (size_t)p.n_layers * sizeof(double) + (sh->warp_small ? TrackCache<kWarpTracksSmall>::kBytes : TrackCache<kWarpTracks>::kBytes);
-  const void* warps = sh->warp_small ? (const void*)k_loop_warps<kWarpTracksSmall> : (const void*)k_loop_warps<kWarpTracks>;
+  for (sh->warp_variant = 0; sh->warp_variant < kWarpVariants; ++sh->warp_variant) {
+    cudaFuncAttributes fa{};
+    e = cudaFuncGetAttributes(&fa, warp_kernel(sh->warp_variant).fn);
+    if (e != cudaSuccess) return e;
+    sh->warp_smem = warp_kernel(sh->warp_variant).bytes + stat + (size_t)p.n_layers * sizeof(double);
+    if (fa.sharedSizeBytes + sh->warp_smem <= (size_t)max_smem || sh->warp_variant == kWarpVariants - 1) break;
+  }
+  const void* warps = warp_kernel(sh->warp_variant).fn;
   e = cudaFuncSetAttribute(warps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh->warp_smem);
   if (e != cudaSuccess) return e;
   sh->tile_grid = occupancy_grid((const void*)k_fill_step, kTile, stat, sms, (int)p.n_tiles);
@@ -2025,7 +2043,7 @@ cudaError_t configure_kernels(const Params& p, int block, LaunchShape* sh) {
   if (e != cudaSuccess) return e;
   if (nb_async < nb) nb = nb_async;
   int nb_warps = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb_warps, warps, kWarpThreads, sh->warp_smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb_warps, warps, warp_kernel(sh->warp_variant).threads, sh->warp_smem);
   if (e != cudaSuccess) return e;
   if (nb_warps < nb) nb = nb_warps;
   sh->loop_grid = (nb < 1 ? 1 : nb) * sms;
@@ -2098,8 +2116,8 @@ void launch_async_prepare(const Params& p, cudaStream_t s) { k_async_prepare<<<2
 cudaError_t launch_loop_async(const Params& p, const LaunchShape& sh, cudaStream_t s) {
   void* args[] = {const_cast<Params*>(&p)};
   if (p.policy == POLICY_LOCAL && p.async_warps) {
-    const void* fn = sh.warp_small ? (const void*)k_loop_warps<kWarpTracksSmall> : (const void*)k_loop_warps<kWarpTracks>;
-    return cudaLaunchCooperativeKernel(fn, dim3(sh.loop_grid), dim3(kWarpThreads), args, sh.warp_smem, s);
+    const WarpKernel k = warp_kernel(sh.warp_variant);
+    return cudaLaunchCooperativeKernel(k.fn, dim3(sh.loop_grid), dim3(k.threads), args, sh.warp_smem, s);
   }
   return cudaLaunchCooperativeKernel((const void*)k_loop_async, dim3(sh.loop_grid), dim3(kTile), args, sh.static_smem,
                                      s);

@@ -950,7 +950,17 @@ constexpr int kAnyPieceWarps = 2;
 // job that runs beside them (10,000 x 10 GeV without the first condition 3.3
 // -> 4.0 ms).
 constexpr int kBaseWarps = 8, kWarpThreads = 512;
-constexpr unsigned kHelpWaiting = 64, kManyLive = 640;
+constexpr unsigned kHelpWaiting = 64;
+// kManyLive by the block's entries: 640 of 1,024 and 400 of 512, above the 186
+// tracks that may sit in part-filled pieces (6 materials, 512 entries, 30,000 x
+// 3 GeV: 4.85 ms without such a number, 4.71 with 400, 4.78 with 320; 10,000 x
+// 10 GeV in 4 T: 3.11, 3.16 and 3.29 ms). Of 256 entries nothing is left
+// between: there no block holds many tracks, and the helpers are not launched
+// (8 materials, 800 layers, 30,000 x 3 GeV: 16.6 ms, and 20.0 with 205).
+template <int kCap>
+constexpr unsigned kManyLive = kCap == 1024 ? 640u : (kCap == 512 ? 400u : ~0u);
+template <int kCap>
+constexpr int kThreads = kCap >= 512 ? kWarpThreads : 32 * kBaseWarps;
 // A block with tracks waiting looks at the buffer this often at most (~2 us).
 constexpr unsigned kLookCycles = 4000;
 // Live tracks a block fills itself up to from the buffer while no full piece
@@ -958,9 +968,10 @@ constexpr unsigned kLookCycles = 4000;
 // kFillLeast (a least of 32 put a small event's tracks on one block: 12
 // particles 0.79 -> 0.69 ms with 2).
 constexpr float kFillShare = 0.75f, kFillLeast = 2.0f;
-// Entries of a block's track store: 1,024, or 256 where the tables of many
-// materials leave no room for more.
-constexpr int kWarpTracks = 1024, kWarpTracksSmall = 256;
+// Entries of a block's track store: the most that fit beside the tables (1,024
+// with up to five materials, 512 up to eight, 256 where the planes and materials
+// of several hundred layers take the rest).
+constexpr int kWarpTracks = 1024, kWarpTracksMid = 512, kWarpTracksSmall = 256;
 
 // Warp sums of the per-lane counts since the last flush (32-bit sums), added
 // to the device counters by lane 0. Ended tracks are counted after a fence,
@@ -1020,7 +1031,7 @@ static __device__ __noinline__ bool idle_poll(const Params& p, bool empty, unsig
 // them, before any initializer unless the buffer is full. A block that runs out
 // of entries while the buffer is full parks tracks too (park_waiting).
 template <int kCap>
-__global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
+__global__ void __launch_bounds__(kThreads<kCap>, 1) k_loop_warps(Params p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TrackCache<kCap> tc{smem_raw};
   const SharedStatic ss = carve_static(p, smem_raw + TrackCache<kCap>::kBytes);
@@ -1120,7 +1131,7 @@ __global__ void __launch_bounds__(kWarpThreads, 1) k_loop_warps(Params p) {
     if (lane == 0)
       flags = (*reinterpret_cast<volatile unsigned*>(&w.exit) != 0u ? 1u : 0u) |
               (*reinterpret_cast<volatile unsigned*>(&s_drain) != 0u ? 2u : 0u) |
-              (*reinterpret_cast<volatile unsigned*>(&w.live) >= kManyLive ? 4u : 0u) |
+              (*reinterpret_cast<volatile unsigned*>(&w.live) >= kManyLive<kCap> ? 4u : 0u) |
               (*reinterpret_cast<volatile unsigned*>(&s_deferred) != 0u ? 8u : 0u);
     flags = __shfl_sync(0xffffffffu, flags, 0);
     const bool drain = (flags & 3u) != 0u, many = (flags & 4u) != 0u, full_buffer = (flags & 8u) != 0u;

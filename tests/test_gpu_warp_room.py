@@ -68,3 +68,23 @@ def test_more_live_tracks_than_entries_at_the_start_and_a_full_buffer(n_material
         hist, edep = ctx.read_history(0, n)
         tally = {0: ctx.read_tallies(0)}
     check(prob.replace(n_slots=1 << 15), prim, hist, edep, tally)
+
+
+@pytest.mark.parametrize("n_materials,n_periods", [(5, 52), (5, 53), (6, 13), (8, 82), (8, 83), (8, 128)])
+def test_as_many_entries_as_fit_beside_the_tables(n_materials, n_periods):
+    """Worlds on both sides of the lines between 1,024, 512 and 256 entries
+    (261 layers of five materials, 658 of eight), four blocks with more tracks
+    than the number from which on they take full pieces only."""
+    n = 3000
+    prob = world(n_materials, init_capacity=1 << 18, history_capacity=n).replace(
+        n_periods=n_periods, layer_thickness=[0.1 if i % 2 == 0 else 0.25 for i in range(n_materials)])
+    prim = wl.electron_beam(n, 100.0, patch_half=5.0)
+    with binding.Context(prob) as ctx:
+        ctx.set_grid_blocks(4)
+        ctx.add_events(prim)
+        ctx.run_events(binding.LOOP_ASYNC)
+        s = ctx.stats()
+        assert s["alive"] == 0 and s["queued"] == 0
+        hist, edep = ctx.read_history(0, n)
+        tally = {0: ctx.read_tallies(0)}
+    check(prob, prim, hist, edep, tally)
