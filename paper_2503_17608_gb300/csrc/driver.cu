@@ -89,7 +89,11 @@ celer_status fail(celer_ctx* ctx, celer_status s, const std::string& msg) {
   return s;
 }
 
+// A failed call of the library: its status, and nothing of it left for the next
+// call of any context on this thread to report (the launches are checked by the
+// runtime's last error).
 celer_status cuda_fail(celer_ctx* ctx, cudaError_t e, const char* where) {
+  cudaGetLastError();
   std::string m = std::string(where) + ": " + cudaGetErrorString(e);
   return fail(ctx, CELER_ERR_CUDA, m);
 }
