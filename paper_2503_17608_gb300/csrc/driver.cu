@@ -179,6 +179,28 @@ void timed(celer_ctx* ctx, cudaStream_t s, int kid, F&& launch, bool allow_timin
   cudaEventRecord(ctx->t_stop[i], s);
 }
 
+// A caller's buffer of n doubles as kernels can write it: aligned, and pinned
+// with one run of device addresses from the first page to the last (memory may
+// be pinned by parts). Null if it is not: it is copied to then.
+double* mapped_rows(double* host, uint64_t n) {
+  if (reinterpret_cast<uintptr_t>(host) % sizeof(double) != 0) return nullptr;
+  unsigned char* const first = reinterpret_cast<unsigned char*>(host);
+  const uint64_t bytes = n * sizeof(double);
+  unsigned char* dev = nullptr;
+  for (uint64_t at = 0;; at = std::min<uint64_t>(at + 4096, bytes - 1)) {
+    cudaPointerAttributes pa{};
+    if (cudaPointerGetAttributes(&pa, first + at) != cudaSuccess) {
+      cudaGetLastError();  // not a CUDA pointer
+      return nullptr;
+    }
+    if (pa.type != cudaMemoryTypeHost || !pa.devicePointer) return nullptr;
+    unsigned char* const d = static_cast<unsigned char*>(pa.devicePointer);
+    if (at == 0) dev = d;
+    if (d != dev + at) return nullptr;
+    if (at == bytes - 1) return reinterpret_cast<double*>(dev);
+  }
+}
+
 // One step iteration as a sequence of launches on stream s. Phase-merged:
 // fill + step limit (+ bookkeeping), scatter, along-step + interactions (+
 // end of iteration). Per action (split_actions), as in the paper's loop over
@@ -978,13 +1000,8 @@ celer_status celer_set_hit_readout(celer_ctx* ctx, int mode, double* host_hits, 
   ctx->hit_mode = mode;
   ctx->h_hits = mode ? host_hits : nullptr;
   ctx->hits_mapped = nullptr;
-  if (mode == 1 && (uint64_t)ctx->p.max_events * (uint64_t)ctx->p.n_bins <= kMappedHits) {
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, host_hits) != cudaSuccess)
-      cudaGetLastError();  // not a CUDA pointer: copied
-    else if (at.type == cudaMemoryTypeHost && at.devicePointer)
-      ctx->hits_mapped = static_cast<double*>(at.devicePointer);
-  }
+  const uint64_t rows = (uint64_t)ctx->p.max_events * (uint64_t)ctx->p.n_bins;
+  if (mode == 1 && rows <= kMappedHits) ctx->hits_mapped = mapped_rows(host_hits, rows);
   return CELER_OK;
 }
 
