@@ -732,13 +732,15 @@ struct BlockWords {
 };
 __device__ __forceinline__ unsigned block_word(const unsigned& a) { return *reinterpret_cast<const volatile unsigned*>(&a); }
 
-// The next chunk with parked tracks, if as many entries are free: its index (or
-// ~0), its parked tracks in `take`, the first of the free entries claimed for
-// them in f0. While the buffer is full (moving_only) the tracks whose
+// The parked tracks of the next chunk that has any, if as many entries are free:
+// each lane's slot (or ~0), their number in `take`, the first of the free entries
+// claimed for them in f0. While the buffer is full (moving_only) the tracks whose
 // interactions wait for room in it stay where they are. The tracks are marked,
 // so that the warp can load them without the block's fill lock, which lane 0
-// holds and this gives up. The whole warp calls it. (One lane looking at the
-// chunk's slots in turn: a run that starts with 140,000 tracks, 0.9 -> 2.0 ms.)
+// holds and this gives up; the lanes know theirs, since others of the chunk may
+// be marked by another warp meanwhile. The whole warp calls it. (One lane looking
+// at the chunk's slots in turn: a run that starts with 140,000 tracks, 0.9 -> 2.0
+// ms.)
 static __device__ __noinline__ uint32_t claim_parked_chunk(const Params& p, BlockWords& w, int bid, int nb, uint32_t n_own,
                                                            bool moving_only, unsigned& take, unsigned& f0) {
   const unsigned lane = threadIdx.x & 31u;
@@ -749,11 +751,11 @@ static __device__ __noinline__ uint32_t claim_parked_chunk(const Params& p, Bloc
   }
   m = __shfl_sync(0xffffffffu, m, 0);
   free_now = __shfl_sync(0xffffffffu, free_now, 0);
-  uint32_t g = 0xFFFFFFFFu;
+  uint32_t mine = 0xFFFFFFFFu;
   unsigned next = m;  // no parked track waits in a chunk before it
   take = 0;
   for (; m < n_own; ++m) {
-    const uint32_t at = (uint32_t)bid + (uint32_t)nb * m, slot = at * 32u + lane;
+    const uint32_t slot = ((uint32_t)bid + (uint32_t)nb * m) * 32u + lane;
     volatile uint8_t* status = p.trk.status + slot;
     const uint8_t st = slot < p.n_slots ? *status : (uint8_t)VACANT;
     const bool parked = st == ALIVE || (st == DEFERRED && !moving_only);
@@ -762,9 +764,11 @@ static __device__ __noinline__ uint32_t claim_parked_chunk(const Params& p, Bloc
     if (cnt > free_now) break;
     if (next == m && !left) next = m + 1u;
     if (cnt > 0) {
-      if (parked) *status = st | CLAIMED;
+      if (parked) {
+        *status = st | CLAIMED;
+        mine = slot;
+      }
       take = cnt;
-      g = at;
       break;
     }
   }
@@ -780,7 +784,7 @@ static __device__ __noinline__ uint32_t claim_parked_chunk(const Params& p, Bloc
   __threadfence_block();
   __syncwarp();
   if (lane == 0) atomicExch(&w.filling, 0u);
-  return g;
+  return mine;
 }
 
 // The tracks still live at the end of a run back into the block's slots:
@@ -1199,7 +1203,7 @@ __global__ void __launch_bounds__(kThreads<kCap>, 1) k_loop_warps(Params p) {
     // all SMs, many keep every block's pieces full
     unsigned take = 0, f0 = 0;
     unsigned long long first = 0;
-    uint32_t load_chunk = 0xFFFFFFFFu;  // a chunk of parked tracks to load
+    uint32_t load_slot = 0xFFFFFFFFu;  // the lane's parked track to load
     constexpr unsigned kParked = 0xFFFFFFFFu;
     // (interactions wait for buffer space: entries must be taken whatever the
     // target, or no block would make room for another)
@@ -1263,7 +1267,7 @@ __global__ void __launch_bounds__(kThreads<kCap>, 1) k_loop_warps(Params p) {
         }
       }
       take = __shfl_sync(0xffffffffu, take, 0);
-      if (take == kParked) load_chunk = claim_parked_chunk(p, w, bid, nb, n_own, full_buffer, take, f0);
+      if (take == kParked) load_slot = claim_parked_chunk(p, w, bid, nb, n_own, full_buffer, take, f0);
     }
     unsigned c = kNoEntry;
     int out = W_NONE;
@@ -1274,16 +1278,12 @@ __global__ void __launch_bounds__(kThreads<kCap>, 1) k_loop_warps(Params p) {
     if (take > 0) {
       first = __shfl_sync(0xffffffffu, first, 0);
       f0 = __shfl_sync(0xffffffffu, f0, 0);
-      load_chunk = __shfl_sync(0xffffffffu, load_chunk, 0);
-      if (load_chunk != 0xFFFFFFFFu) {
-        const uint32_t slot = load_chunk * 32u + (uint32_t)lane;
+      const unsigned loads = __ballot_sync(0xffffffffu, load_slot != 0xFFFFFFFFu);
+      if (loads) {
         __threadfence_block();
-        const bool live =
-            slot < p.n_slots && (*reinterpret_cast<volatile uint8_t*>(p.trk.status + slot) & CLAIMED) != 0u;
-        const unsigned bal = __ballot_sync(0xffffffffu, live);
-        if (live) {
-          c = pop_entry(p, tc, W_FREE, f0 + (unsigned)__popc(bal & lt));
-          if (c != kNoEntry) out = load_entry(p, tc, slot, c);
+        if (load_slot != 0xFFFFFFFFu) {
+          c = pop_entry(p, tc, W_FREE, f0 + (unsigned)__popc(loads & lt));
+          if (c != kNoEntry) out = load_entry(p, tc, load_slot, c);
         }
         // (they were counted alive already)
       } else {
@@ -1379,8 +1379,9 @@ __global__ void __launch_bounds__(kThreads<kCap>, 1) k_loop_warps(Params p) {
         atomicSub(&p.event_live[row_of(p, ev)], 1u);
         if (m & kMetaStored) {
           const uint32_t slot = tc.home(c);
-          p.trk.status[slot] = VACANT;
           p.trk.action[slot] = A_NONE;
+          __threadfence_block();  // park_waiting may take the slot as soon as it is vacant
+          *reinterpret_cast<volatile uint8_t*>(p.trk.status + slot) = VACANT;
           atomicAdd(&p.vacant[slot >> 5], 1u);
           atomicAdd(&p.tile_vacant[slot >> 8], 1u);
         }
