@@ -116,15 +116,14 @@ __device__ __forceinline__ void end_async_block(const Params& p, int nb, unsigne
 // chunks with no grid barrier. At the start of a pass a block claims
 // written entries on an availability count (atomic, undone if short) and
 // takes their indices from the head: ceil(queued / blocks) or enough to hold
-// kAsyncFill live tracks, at most its vacant slots. Secondaries are reserved
-// at the tail against the current head, and each entry's state word orders
+// kAsyncFill live tracks, at most its vacant slots. Secondaries are reserved on
+// the count of free entries (reserve_entries), and each entry's state word orders
 // its writer and its reader. A track's steps and draws do not depend
 // on where or when it runs (its random stream is keyed by its own id), so
 // histories are those of the synchronous loops; only the tally summation
 // order differs. The run ends when every track taken from the buffer has
 // ended (finished reaches tail), or, with an iteration budget, when every
-// block has run that many passes or holds no track (warp_queue_loop: has
-// drained). Every wait is bounded: a block with nothing to do polls, and if
+// block has run that many passes or holds no track. Every wait is bounded: a block with nothing to do polls, and if
 // no track anywhere steps for ~1 s it sets ERR_NO_PROGRESS and the abort
 // word; all blocks leave at their next pass. The last block to leave adds
 // the most passes (pieces) any block ran to the iteration count.

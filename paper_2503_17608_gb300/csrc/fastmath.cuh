@@ -105,19 +105,28 @@ inline void build_math_table(double* out) {
 #ifdef __CUDACC__
 // ---- quotient, square root and reciprocal square root
 //
-// From the hardware's approximation (rcp.approx.ftz.f64, rsqrt.approx.ftz.f64:
-// documented relative error about 2^-23) by Newton-Raphson steps that end in
-// a correction by the exact residual (P. W. Markstein, "Computation of
-// elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
-// Dev. 34, 1990): the error before the last rounding is below 2^-64, so the
-// quotient and the square root are the correctly rounded ones but for rare
-// near-ties, and the reciprocal square root is within 1 ulp.
+// From the hardware's approximation (rcp.approx.ftz.f64, rsqrt.approx.ftz.f64)
+// by Newton-Raphson steps that end in a correction by the exact residual (P. W.
+// Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990). The PTX ISA states no error bound for
+// the approximations; it describes the reciprocal as taking and returning 20 bits
+// of mantissa, so take 2^-19 relative for both. Before its last rounding then
+//  * the reciprocal after one Newton step is within 2^-38, the quotient's and the
+//    reciprocal's correction by it within 2^-76: the rounded result but for
+//    near-ties of that size;
+//  * the square root is within 2^-37 (3/2 e^2) after one step, its correction by
+//    half the approximate reciprocal root within 2^-56: at most one ulp off;
+//  * the reciprocal root's third-order step leaves 5/16 (2 e)^3, 2^-55.
+// Against correctly rounded values the quotient and the reciprocal differ in fewer
+// than 10^-5 of the operands tested and the square root in fewer than 2^-11 of
+// them, by one ulp; the reciprocal root is within one ulp. (The operators' are
+// correctly rounded.)
 //
 // Why not the operators: they cost 8 to 11 FP64 instructions; these cost 5.
 // On sm_103a an FP64 instruction holds the sub-partition's FP64 pipe for 64
-// cycles and takes five instruction slots of code (80 bytes, measured on the
-// size of compiled loops), and the step loops stall on instruction fetch and
-// on that pipe. Operands outside the middle of the exponent range (zeros,
+// cycles, and the step loops stall on that pipe and on instruction fetch (with
+// the kept grid positions and one root per rotation the timed cases became 1.04
+// to 1.12 times as fast). Operands outside the middle of the exponent range (zeros,
 // subnormals, infinities and NaN among them) take the operators, one shared
 // copy of each.
 __device__ __forceinline__ double approx_rcp(double b) {
@@ -141,7 +150,7 @@ static __device__ __noinline__ double quot_any(double n, double b) { return n / 
 static __device__ __noinline__ double sqrt_any(double x) { return sqrt(x); }
 static __device__ __noinline__ double rsqrt_any(double x) { return rsqrt(x); }
 
-// 1 / b to about 2^-46 relative: one Newton step.
+// 1 / b to 2^-38 relative or better: one Newton step.
 __device__ __forceinline__ double rough_rcp(double b) {
   const double r = approx_rcp(b);
   return fma(r, fma(-b, r, 1.0), r);

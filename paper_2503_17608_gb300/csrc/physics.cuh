@@ -289,7 +289,7 @@ static __device__ __noinline__ RkState rk_substeps_move(double kappa, double s, 
   uy = V;
   return RkState{x, y, z, ux, uy};
 }
-// (called, not inlined: 14 KB of code that runs with the substep cap only)
+// (called, not inlined: it runs with the substep cap only)
 __device__ __forceinline__ void rk_move(double kappa, double s, int n, double& x, double& y, double& z, double& ux,
                                         double& uy, double uz) {
   const RkState r = rk_substeps_move(kappa, s, n, RkState{x, y, z, ux, uy}, uz);
@@ -365,8 +365,8 @@ static __device__ __noinline__ double helix_side_distance(Curvature c, double x,
 //    within 2^-22 + |x| 2^-23 (below 2^-18.5 for |x| <= 15), e^x - 1 is taken
 //    from a five-term series below |x| = 1/8 (truncation 2^-24) and from e^x
 //    above (2^-19). They take a third of the instructions of the rounded
-//    library forms (sampler 10.6 -> 6.6 KB of code; asynchronous loop, 4 T
-//    calorimeter, 10,000 x 10 GeV 3.82 -> 3.50 ms, 100,000 27.6 -> 25.4 ms);
+//    library forms (asynchronous loop, 4 T calorimeter, 10,000 x 10 GeV 3.82 ->
+//    3.50 ms, 100,000 27.6 -> 25.4 ms);
 //  * a decision is taken in FP32 only if the two sides differ by more than
 //    kFilterMargin = 2^-12 relative, far above both error bounds, so both
 //    evaluations take the same decision; otherwise (probability ~2^-11 per

@@ -65,16 +65,20 @@ __device__ __forceinline__ void flush_counter(unsigned long long* dst, unsigned 
 // Entry i of the buffer (stored at i & ring_mask) carries a state word: with
 // lap = i / capacity, 2 lap means free for the writer of i, 2 lap + 1 written
 // and not yet read, 2 lap + 2 read (free for the writer of i + capacity).
-// A writer reserves i on the tail only while i < head + capacity, with the
-// head read just before: by compare-and-swap, or by one atomic add while the
-// room exceeds what every thread of the grid could reserve at once (should
-// the buffer still fill within that window, the writer's wait below for the
-// entry's reader is bounded like every other). So the reader of
-// i - capacity has claimed its entry already, and every wait is for a claim
-// or reservation that the other side completes without waiting on the
-// waiter: reads and writes follow their claims and reservations directly.
-// Readers claim written entries on an availability count (avail) before
-// taking their indices from the head, so the head never passes the tail.
+// The count of free entries (ctl->room) goes with it. A reader claims written
+// entries on an availability count (avail), takes their indices from the head,
+// so that the head never passes the tail, and adds them to room after that. A
+// writer takes its entries off room before it moves the tail (reserve_entries;
+// what room is short of goes back). So the tail never passes head + capacity:
+// the reader of i - capacity has claimed it before i is reserved.
+// Waits: the reader of i waits for its writer, which has reserved it; the writer
+// of i waits for the reader of i - capacity, which has claimed it. Neither side
+// does anything else in between that could wait: a writer writes what it has
+// reserved, a warp reads its fill, and a block pass reads all it has claimed
+// before its first step (fill_block). A warp's lanes end their waits together, so
+// a wait also lasts for the other entries of the same claim or reservation, some
+// tens of indices away. Every chain of waits thus runs to lower indices, by about
+// a capacity every second link, and ends.
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* a) {
   unsigned v;
   asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
@@ -1051,14 +1055,13 @@ __device__ __forceinline__ bool photoelectric_one(const Params& p, uint32_t slot
 // the track keeps its state and draw counter, so the interaction replays
 // identically in a later iteration.
 // The lanes of a group are the active ones of the warp, each wanting n = 0, 1
-// or 2 entries; two ballots give every lane its place (a generic scan over the
-// group compiled to 12 KB of code at each of the three call sites, this form
-// to 1 KB and the tight case to one called function). With the other cold
-// code taken out of line (side planes, Runge-Kutta substeps, the row's
-// division) and the buffer's records moved in 16-byte parts, the loops fetch
-// fewer instructions: 4 T calorimeter with the charge partition, persistent
-// loop, 10.26 -> 9.32 ms; 1 GeV calorimeter sorted by action and type 4.85 ->
-// 4.37 ms; asynchronous loop 1.30 -> 1.27 ms.
+// or 2 entries; two ballots give every lane its place (instead of a generic scan
+// over the group at each of the three call sites), and the tight case is one
+// called function. With the other cold code taken out of line (side planes,
+// Runge-Kutta substeps, the row's division) and the buffer's records moved in
+// 16-byte parts, the loops fetch fewer instructions: 4 T calorimeter with the
+// charge partition, persistent loop, 10.26 -> 9.32 ms; 1 GeV calorimeter sorted
+// by action and type 4.85 -> 4.37 ms; asynchronous loop 1.30 -> 1.27 ms.
 static __device__ __noinline__ bool reserve_tight(const Params& p, unsigned group, unsigned end, unsigned prefix,
                                                   unsigned n, unsigned long long& base) {
   Ctl* c = p.ctl;
@@ -1088,11 +1091,11 @@ static __device__ __noinline__ bool reserve_tight(const Params& p, unsigned grou
 // In the asynchronous loops, where readers move the head meanwhile, a group
 // takes its entries off the count of free ones (ctl->room) first: one atomic
 // tells how many it got, the lanes that these are too few for give theirs
-// back, and the tail moves by what is left. No group waits for another's. (A
-// compare-and-swap on the tail while the room was short let one group at a
-// time through. Before and after: 60,000 x 100 MeV with a buffer of 2^19
-// entries 7.4 and 2.7 ms, 20,000 x 1 GeV with 2^17 29 and 2.7 ms; 2.7 and 2.5
-// ms with 2^20.)
+// back, and the tail moves by what is left. No group waits for another's, as
+// with a compare-and-swap on the tail while the room is short (per-warp loop with
+// one and with the other: 60,000 x 100 MeV with a buffer of 2^19 entries 7.4 and
+// 2.7 ms, 20,000 x 1 GeV with 2^17 29 and 2.7 ms, the former with 2^20 2.7 and 2.5;
+// the loop before it, with its swaps, took 4.95 and 12.3 ms).
 // (reserve_entries holds the case of room for all; this is what follows for a
 // group that asked for `total` when only `got` were free.)
 static __device__ __noinline__ bool reserve_rest(const Params& p, unsigned group, unsigned total, long long got,
